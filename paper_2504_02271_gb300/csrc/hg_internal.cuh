@@ -84,10 +84,11 @@ void launch_wait_flag(const int32_t* flag, int64_t limit_ns, int* err, cudaStrea
 void launch_check_ptr(const int64_t* e_ptr, int32_t ne, int64_t nnz, int* err, cudaStream_t s);
 void launch_validate_rows(const DevGraph& g, int32_t* esize, int32_t* vdeg, int* err,
                           cudaStream_t s);
-void launch_scatter(const DevGraph& g, int32_t* cursor, int32_t* v_idx, cudaStream_t s);
+void launch_scatter(const DevGraph& g, int32_t* cursor, int32_t* v_idx, const int* err,
+                    cudaStream_t s);
 // cand[i] = sum_{v in e_i} (|E_v| - 1); also bucket rows by cand into lists
 void launch_candidates(const DevGraph& g, int64_t* cand, unsigned long long* max_cand,
-                       int32_t* max_size, cudaStream_t s);
+                       int32_t* max_size, const int* err, cudaStream_t s);
 
 // k_dense.cu: heavy x heavy omega on the tensor cores
 struct DenseInfo {

@@ -33,9 +33,10 @@ __global__ void k_add_member_base(int64_t* __restrict__ e_ptr, int32_t ne,
 }
 
 // Member-local vertex ids -> union ids (v + m_voff[m]); ids outside [0, |V_m|) set DE_RANGE.
-// Runs after the row pointers were checked, so every row range lies in [0, nnz).
+// Works only after the row pointers were checked, so every row range lies in [0, nnz).
 __global__ void k_localize(DevGraph g, const int32_t* __restrict__ m_voff, int32_t* __restrict__ e_idx,
                            int* __restrict__ err) {
+  if (*(volatile const int*)err != DE_OK) return;
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   for (int32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < g.ne; i += warps) {

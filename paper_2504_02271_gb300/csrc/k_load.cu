@@ -44,10 +44,18 @@ __global__ void k_wait_flag(const int32_t* flag, int64_t limit_ns, int* __restri
   dev_fail(err, DE_TIMEOUT);
 }
 
+// The load's kernels follow one another without a look from the host: each does nothing
+// once an earlier one has recorded an error (a later kernel relies on what the earlier ones
+// checked).
+__device__ __forceinline__ bool failed(const int* err) {
+  return *(volatile const int*)err != DE_OK;
+}
+
 // Row checks (ascending, distinct, in range), |e_i| and vertex degrees |E_v|.
-// Runs only after k_check_ptr passed, so every row range lies inside [0, nnz).
+// Works only after k_check_ptr passed, so every row range lies inside [0, nnz).
 __global__ void k_validate_rows(DevGraph g, int32_t* __restrict__ esize,
                                 int32_t* __restrict__ vdeg, int* __restrict__ err) {
+  if (failed(err)) return;
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   for (int32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < g.ne; i += warps) {
@@ -73,7 +81,9 @@ __global__ void k_validate_rows(DevGraph g, int32_t* __restrict__ esize,
   }
 }
 
-__global__ void k_scatter(DevGraph g, int32_t* __restrict__ cursor, int32_t* __restrict__ v_idx) {
+__global__ void k_scatter(DevGraph g, int32_t* __restrict__ cursor, int32_t* __restrict__ v_idx,
+                          const int* __restrict__ err) {
+  if (failed(err)) return;
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   for (int32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < g.ne; i += warps) {
@@ -90,7 +100,8 @@ __global__ void k_scatter(DevGraph g, int32_t* __restrict__ cursor, int32_t* __r
 // thread per row (rows are short); maxima reduced per warp before their atomics.
 __global__ void k_candidates(DevGraph g, int64_t* __restrict__ cand,
                              unsigned long long* __restrict__ max_cand,
-                             int32_t* __restrict__ max_size) {
+                             int32_t* __restrict__ max_size, const int* __restrict__ err) {
+  if (failed(err)) return;
   const int lane = threadIdx.x & 31;
   unsigned long long my_max = 0;
   int32_t my_size = 0;
@@ -148,17 +159,18 @@ void launch_validate_rows(const DevGraph& g, int32_t* esize, int32_t* vdeg, int*
   k_validate_rows<<<grid_for(g.ne, 8), 256, 0, s>>>(g, esize, vdeg, err);
 }
 
-void launch_scatter(const DevGraph& g, int32_t* cursor, int32_t* v_idx, cudaStream_t s) {
+void launch_scatter(const DevGraph& g, int32_t* cursor, int32_t* v_idx, const int* err,
+                    cudaStream_t s) {
   if (g.ne == 0) return;
   note_launch();
-  k_scatter<<<grid_for(g.ne, 8), 256, 0, s>>>(g, cursor, v_idx);
+  k_scatter<<<grid_for(g.ne, 8), 256, 0, s>>>(g, cursor, v_idx, err);
 }
 
 void launch_candidates(const DevGraph& g, int64_t* cand, unsigned long long* max_cand,
-                       int32_t* max_size, cudaStream_t s) {
+                       int32_t* max_size, const int* err, cudaStream_t s) {
   if (g.ne == 0) return;
   note_launch();
-  k_candidates<<<grid_for(g.ne, 256), 256, 0, s>>>(g, cand, max_cand, max_size);
+  k_candidates<<<grid_for(g.ne, 256), 256, 0, s>>>(g, cand, max_cand, max_size, err);
 }
 
 }  // namespace hg
