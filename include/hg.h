@@ -88,9 +88,9 @@ typedef struct hg_tuning {
   int32_t dense_max_count; /* cap on the size of the dense set (0 = 1% of |E|) */
   int32_t close_mode;      /* step two team shape: 0 = by out-degree and |e_u| (warp
                               teams where they fit), 1 = global-table teams for every
-                              hyperedge, 2 = warp and block teams build their tables,
-                              then hand every hyperedge over to the global-table teams
-                              (the path a team whose cuckoo stash overflows takes);
+                              hyperedge, 2 = warp and bit-row teams build their
+                              tables, then hand every hyperedge over to the global-table
+                              teams (the path a team whose tables overflow takes);
                               counts do not depend on it */
   int32_t orient_exact;    /* 1 = oriented rows in an exact layout (W entries, one extra
                               counting pass); 0 = room for deg(i) per row (2W entries)
@@ -100,7 +100,7 @@ typedef struct hg_tuning {
                                holds: 512 in the packed layout, 256 otherwise; 32..512,
                                capped at that largest) */
   int32_t warp_team_max;   /* step two: largest out-degree closed by a one-warp team; larger
-                              ones take block teams (0 = 256; 64, 128 or 256) */
+                              ones take bit-row teams (0 = 256; 64, 128 or 256) */
   int32_t reserved[2];
 } hg_tuning;
 
@@ -297,13 +297,13 @@ hg_status hg_clustering_coeff(hg_graph* g, const double eps[20], double* cc,
  *   out_entries  entries of the teams' own out-lists out(u) (= oriented wedges
  *                of hyperedges with out-degree >= 2);
  *   teams        hyperedges u that owned a closing team (out-degree >= 2);
- *   bucket_*     the same per team shape: warp teams for out-degree <= 64, <= 128,
- *                <= 256 (indices 0-2); block teams with shared-memory tables for <= 1024,
- *                <= 2048 and <= 6144 (<= 4096 when omega or ids need the 8-byte row
- *                layout) (3-5); block teams with global-memory tables for hyperedges of
- *                more than 32 vertices with out-degree <= 4096 and for what the other
- *                teams hand over (6); thread-block clusters sharing global-memory tables
- *                for larger out-degrees (7).
+ *   bucket_*     the same per team shape, by out-degree and |e_u|: out-degree <= 64,
+ *                <= 128, <= 256 (indices 0-2), <= 1024, <= 2048 and <= 6144 (<= 4096 when
+ *                omega or ids need the 8-byte row layout) (3-5); hyperedges of more than
+ *                32 vertices with out-degree <= 4096 and what teams hand over (6); larger
+ *                out-degrees (7).  The counters are those of the list walk (one probe per
+ *                entry of out(v)), whichever kernel closes the hyperedge: bit rows answer
+ *                the same probes without the walk.
  */
 typedef struct hg_close_stats {
   uint64_t probes;

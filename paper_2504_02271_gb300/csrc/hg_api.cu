@@ -38,14 +38,16 @@ struct Small {
   int err;
   int32_t pad0;
   int32_t counters[16];       // work-fetch counters
-  int32_t bucket_count[16];   // [0..2] wedge buckets, [3] handed-over teams, [4..9] close buckets
+  int32_t bucket_count[4];    // [0..2] wedge buckets
+  int32_t list_count[kLists];        // closure: owners per list ([kListOver]: handed over)
+  int32_t label_count[kCloseBuckets];   // closure: owners per team shape
   unsigned long long wc;      // inclusion-type wedges
   unsigned long long max_cand;
   int32_t max_size;
   int32_t pad1;
   unsigned long long deg_stats[3];   // sum C(deg,2), max deg, sum deg
   unsigned long long out_stats[3];   // sum C(d+,2), max d+, sum d+
-  unsigned long long wide_max[2];    // close bucket 3: max d+, max |e_u|
+  unsigned long long close_max[6];   // see CloseLists::maxima
   unsigned long long hist[128];      // closure: labelled region masks; samplers: bins 0..20
   unsigned long long work[kCloseBuckets][3];   // closure per team shape: probes, E_y entries, out-entries
   unsigned long long found;                    // triples of hg_enumerate_pattern
@@ -87,6 +89,9 @@ struct hg_graph {
   int warp_team_max = 256;   // of the last build (step two routes teams by it)
   hg_tuning tuned{};         // hg_autotune's choice, used by builds given no tuning
   bool has_tuned = false;
+  uint4* rec = nullptr;      // DevGraph::rec, osum
+  int32_t* osum = nullptr;
+  int32_t* dsum = nullptr;
   uint64_t two_w = 0;
   bool built = false;
   hg_wedge_stats stats{};
@@ -270,6 +275,10 @@ DevGraph dev_graph(const hg_graph* g) {
   d.v_idx = g->v_idx;
   d.m_eoff = g->m_eoff;
   d.nm = g->nm;
+  d.rec = g->rec;
+  d.osum = g->osum;
+  d.dsum = g->dsum;
+  d.cand = g->cand;
   return d;
 }
 
@@ -631,6 +640,7 @@ hg_status build_impl(hg_graph* g, const hg_tuning* opt, hg_wedge_stats* out) {
   Small h;
   HG_CUDA(cudaMemsetAsync(g->small, 0, sizeof(Small), s));
   int32_t *rows = nullptr, *cap = nullptr;
+  int2* ds = nullptr;   // (deg, |e|), read by the orientation
   Carver c;
   c.want(g->deg, ne);
   c.want(g->upc, ne);
@@ -641,6 +651,10 @@ hg_status build_impl(hg_graph* g, const hg_tuning* opt, hg_wedge_stats* out) {
   c.want(g->deg_ptr, ne + 1);
   c.want(g->ori.row_ptr, ne + 1);
   c.want(g->ori.dplus, ne);
+  c.want(ds, ne);
+  c.want(g->rec, ne);
+  c.want(g->osum, ne);
+  c.want(g->dsum, ne);
   if (!c.get(g, g->build_blocks)) return HG_ERR_OOM;
   g->mstats = nullptr;
   if (g->nm > 0) {
@@ -690,7 +704,7 @@ hg_status build_impl(hg_graph* g, const hg_tuning* opt, hg_wedge_stats* out) {
   // to an exact layout (a counting pass, its scan, then the filter pass).
   t_begin(g, "wedge_orient");
   scan_i32_to_i64(g->deg, g->deg_ptr, ne, g->scan_tmp, s);
-  reduce_deg_stats(g->deg, ne, g->small->deg_stats, s);
+  launch_deg_stats(g->deg, g->esize, ne, g->small->deg_stats, ds, s);
   t_end(g);
   // 2W, the entries of all rows, is at most the capacity rows' entries; while those are few
   // the oriented rows get that room, and the true 2W comes with the last read
@@ -705,8 +719,8 @@ hg_status build_impl(hg_graph* g, const hg_tuning* opt, hg_wedge_stats* out) {
   int64_t slots = two_w;
   if (exact) {
     t_begin(g, "wedge_orient");
-    launch_filter_rows(0, true, g->cap_ptr, g->deg, g->cap_rows, g->deg, g->ne, g->packed,
-                       nullptr, Oriented{}, g->ori.dplus, s);
+    launch_filter_rows(0, true, g->cap_ptr, g->deg, g->cap_rows, ds, g->ne, g->packed, nullptr,
+                       Oriented{}, g->ori.dplus, nullptr, nullptr, s);
     scan_i32_to_i64(g->ori.dplus, g->ori.row_ptr, ne, g->scan_tmp, s);
     t_end(g);
     HG_TRY(read_total(g, g->ori.row_ptr + ne, &h));
@@ -725,9 +739,9 @@ hg_status build_impl(hg_graph* g, const hg_tuning* opt, hg_wedge_stats* out) {
     if (!g->ori.nbr || !g->ori.omega) return HG_ERR_OOM;
   }
   t_begin(g, "wedge_emit");
-  launch_filter_rows(0, false, g->cap_ptr, g->deg, g->cap_rows, g->deg, g->ne, g->packed,
-                     g->ori.row_ptr, g->ori, exact ? nullptr : g->ori.dplus, s);
-  reduce_deg_stats(g->ori.dplus, ne, g->small->out_stats, s);
+  launch_filter_rows(0, false, g->cap_ptr, g->deg, g->cap_rows, ds, g->ne, g->packed,
+                     g->ori.row_ptr, g->ori, exact ? nullptr : g->ori.dplus, g->osum, g->dsum, s);
+  launch_out_stats(g->ori.dplus, g->e_ptr, g->esize, ne, g->small->out_stats, g->rec, s);
   t_end(g);
   if (g->nm > 0) {
     g->h_mstats.assign(4 * (size_t)g->nm, 0);
@@ -781,8 +795,8 @@ hg_status upper_impl(hg_graph* g) {
     if (!g->up.nbr || !g->up.omega) return HG_ERR_OOM;
   }
   t_begin(g, "upper_emit");
-  launch_filter_rows(1, false, g->cap_ptr, g->deg, g->cap_rows, g->deg, g->ne, g->packed,
-                     g->up_ptr, g->up, nullptr, s);
+  launch_filter_rows(1, false, g->cap_ptr, g->deg, g->cap_rows, nullptr, g->ne, g->packed,
+                     g->up_ptr, g->up, nullptr, nullptr, nullptr, s);
   t_end(g);
   t_begin(g, "upper_sort");
   HG_CUDA(launch_sort_upper(g->up_ptr, g->ne, g->up, g->packed, &g->small->err, s, g->nsm));
@@ -850,8 +864,8 @@ hg_status adv_impl(hg_graph* g) {
   launch_row_index(g->t_ptr, g->ne, g->Wt, g->t_index, s);
   launch_row_index(g->c_ptr, g->ne, g->Wc, g->c_index, s);
   t_begin(g, "full_emit");
-  launch_filter_rows(2, false, g->cap_ptr, g->deg, g->cap_rows, g->deg, g->ne, g->packed,
-                     g->deg_ptr, g->full, nullptr, s);
+  launch_filter_rows(2, false, g->cap_ptr, g->deg, g->cap_rows, nullptr, g->ne, g->packed,
+                     g->deg_ptr, g->full, nullptr, nullptr, nullptr, s);
   t_end(g);
   t_begin(g, "full_sort");
   HG_CUDA(launch_sort_upper(g->deg_ptr, g->ne, g->full, g->packed, &g->small->err, s, g->nsm));
@@ -1051,7 +1065,7 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
   g->counted = g->have_cstats = false;
   const int64_t ne = g->ne;
   Small h;
-  int32_t* lists = alloc_t<int32_t>(g, g->count_blocks, (kCloseBuckets + 1) * ne);  // + overflow
+  int32_t* lists = alloc_t<int32_t>(g, g->count_blocks, kLists * ne);
   if (!lists) return HG_ERR_OOM;
   uint8_t* sel = nullptr;
   if (h_sel) {
@@ -1059,8 +1073,9 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
     if (!sel) return HG_ERR_OOM;
     HG_CUDA(cudaMemcpyAsync(sel, h_sel, (size_t)ne, cudaMemcpyHostToDevice, s));
   }
-  HG_CUDA(cudaMemsetAsync(g->small->bucket_count + 3, 0, sizeof(int32_t) * (1 + kCloseBuckets), s));
-  HG_CUDA(cudaMemsetAsync(g->small->wide_max, 0, sizeof(g->small->wide_max), s));
+  HG_CUDA(cudaMemsetAsync(g->small->list_count, 0,
+                          sizeof(g->small->list_count) + sizeof(g->small->label_count), s));
+  HG_CUDA(cudaMemsetAsync(g->small->close_max, 0, sizeof(g->small->close_max), s));
   HG_CUDA(cudaMemsetAsync(g->small->hist, 0, sizeof(g->small->hist), s));
   HG_CUDA(cudaMemsetAsync(g->small->work, 0, sizeof(g->small->work), s));
   HG_CUDA(cudaMemsetAsync(g->small->counters, 0, sizeof(int32_t) * 16, s));
@@ -1072,53 +1087,80 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
     HG_CUDA(cudaMemsetAsync(g->mhist, 0, sizeof(unsigned long long) * 128 * (size_t)g->nm, s));
     hist = g->mhist;
   }
-  CloseBuckets cb;
-  for (int k = 0; k < kCloseBuckets; ++k) cb.lists[k] = lists + k * ne;
-  cb.count = g->small->bucket_count + 4;
-  int32_t* overflow = lists + kCloseBuckets * ne;
-  int32_t* n_overflow = g->small->bucket_count + 3;
+  CloseLists cl;
+  for (int k = 0; k < kLists; ++k) cl.lists[k] = lists + k * ne;
+  cl.count = g->small->list_count;
+  cl.labels = g->small->label_count;
+  cl.maxima = g->small->close_max;
   DevGraph d = dev_graph(g);
+  TeamRule rule;
+  // the warp teams keep |e_x| in 16 bits: larger hyperedges send everything to the
+  // global-table blocks
+  rule.all_wide = g->close_mode == 1 || g->max_size >= 65536;
+  rule.warp_max = g->warp_team_max;
+  rule.block_max = g->packed ? kBlockMaxPacked : kBlockMaxUnpacked;
+  const int handover = g->close_mode == 2 ? 1 : 0;
   t_begin(g, "close_bucket");
-  // warp tables keep |e_x| in 16 bits: larger hyperedges send everything to block teams
-  launch_bucket_close(d, g->ori, cb, g->small->wide_max,
-                      g->close_mode == 1 || g->max_size >= 65536, g->warp_team_max,
-                      g->packed ? kBlockMaxPacked : kBlockMaxUnpacked, sel, s);
+  launch_bucket_close(d, g->ori, cl, rule, sel, s);
   t_end(g);
   HG_TRY(sync_small(g, &h));
-  int32_t n[kCloseBuckets];
-  for (int k = 0; k < kCloseBuckets; ++k) n[k] = h.bucket_count[4 + k];
-  // block-kernel scratch: any out-degree and |e_u| of bucket 3, and the warp
-  // and block buckets' limits (the largest out-degree of a non-empty one, |e_u| 32) for
-  // hyperedges they hand over
-  int64_t team_dmax = 256;
-  for (int k = 3; k < kWideBucket; ++k)
-    if (n[k] > 0)
-      team_dmax = k < 5 ? int64_t(1024) << (k - 3) : (g->packed ? kBlockMaxPacked : kBlockMaxUnpacked);
-  const int64_t dmax = std::max<int64_t>((int64_t)h.wide_max[0], team_dmax);
-  const int64_t words = std::max<int64_t>(((int64_t)h.wide_max[1] + 31) / 32, 1);
-  int64_t cap = 16;
-  while (cap < 2 * dmax) cap *= 2;
-  void* scratch = dev_alloc(g, g->count_blocks, close_wide_scratch_bytes(cap, words, dmax, g->nsm));
-  if (!scratch) return HG_ERR_OOM;
-  static const char* names[kCloseBuckets] = {"close_warp256",   "close_warp512",
-                                             "close_warp1024",  "close_block2048",
-                                             "close_block4096", "close_block8192",
-                                             "close_wide",      "close_cluster"};
-  for (int k = kCloseBuckets - 1; k >= 0; --k) {
+  int32_t n[kLists];
+  for (int k = 0; k < kLists; ++k) n[k] = h.list_count[k];
+  // scratch of the global-table teams: out-degrees and |e_u| up to the two maxima
+  struct Wide {
+    int64_t cap = 16, words = 1, dmax = 1;
+    void* scratch = nullptr;
+  };
+  auto wide_scratch = [&](unsigned long long dmax, unsigned long long smax, Wide* w) {
+    w->dmax = std::max<int64_t>((int64_t)dmax, 1);
+    w->words = std::max<int64_t>(((int64_t)smax + 31) / 32, 1);
+    while (w->cap < 2 * w->dmax) w->cap *= 2;
+    w->scratch = dev_alloc(g, g->count_blocks,
+                           close_wide_scratch_bytes(w->cap, w->words, w->dmax, g->nsm));
+    return w->scratch != nullptr;
+  };
+  Wide wide;
+  if (n[kListWide] + n[kListCluster] > 0 && !wide_scratch(h.close_max[0], h.close_max[1], &wide))
+    return HG_ERR_OOM;
+  const int64_t slice_dmax = ((int64_t)h.close_max[5] + 15) / 16 * 16;
+  const int64_t slice = bits_slice_bytes(slice_dmax, (int64_t)h.close_max[4]);
+  const int slice_blocks = std::min(n[kListBits + kBitClasses - 1], g->nsm);
+  void* slices = nullptr;
+  if (slice_blocks > 0) {
+    slices = dev_alloc(g, g->count_blocks, (size_t)(slice * slice_blocks));
+    if (!slices) return HG_ERR_OOM;
+  }
+  static const char* names[kLists] = {"close_warp256",  "close_warp512",    "close_warp1024",
+                                      "close_bits64",   "close_bits128",    "close_bits256",
+                                      "close_bits512",  "close_bits1024",   "close_bits_large",
+                                      "close_wide",     "close_cluster",    "close_over"};
+  int32_t* overflow = cl.lists[kListOver];
+  int32_t* n_overflow = cl.count + kListOver;
+  for (int k = kListCluster; k >= 0; --k) {
     if (n[k] <= 0) continue;
     t_begin(g, names[k]);
-    launch_close(k, d, g->ori, g->packed, cb.lists[k], n[k], cb.count + k, cap, words, dmax,
-                 scratch, hist, g->small->work[k], g->small->counters + k, overflow,
-                 n_overflow, g->close_mode == 2 ? 1 : 0, s, g->nsm);
+    if (k >= kListBits && k < kListWide)
+      HG_CUDA(launch_close_bits(k - kListBits, d, g->ori, g->packed, cl.lists[k], n[k],
+                                cl.count + k, slices, slice, slice_dmax, slice_blocks, hist,
+                                &g->small->work[0][0], rule, g->small->counters + k, overflow,
+                                n_overflow, handover, s, g->nsm));
+    else
+      HG_CUDA(launch_close(k, d, g->ori, g->packed, cl.lists[k], n[k], cl.count + k, wide.cap,
+                           wide.words, wide.dmax, wide.scratch, hist,
+                           g->small->work[k == kListCluster ? kClusterBucket
+                                                            : (k == kListWide ? kWideBucket : k)],
+                           g->small->counters + k, overflow, n_overflow, handover, s, g->nsm));
     t_end(g);
   }
   HG_TRY(sync_small(g, &h));
-  const int32_t n_over = h.bucket_count[3];
+  const int32_t n_over = h.list_count[kListOver];
   if (n_over > 0) {
+    Wide over;
+    if (!wide_scratch(h.close_max[2], h.close_max[3], &over)) return HG_ERR_OOM;
     t_begin(g, "close_wide");
-    launch_close(kWideBucket, d, g->ori, g->packed, overflow, n_over, n_overflow, cap, words, dmax,
-                 scratch, hist, g->small->work[kWideBucket], g->small->counters + 8,
-                 overflow, n_overflow, 0, s, g->nsm);
+    HG_CUDA(launch_close(kListOver, d, g->ori, g->packed, overflow, n_over, n_overflow, over.cap,
+                         over.words, over.dmax, over.scratch, hist, g->small->work[kWideBucket],
+                         g->small->counters + kListOver, overflow, n_overflow, 0, s, g->nsm));
     t_end(g);
     HG_TRY(sync_small(g, &h));
   }
@@ -1148,10 +1190,10 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
     g->cstats.out_entries += h.work[k][2];
   }
   for (int k = 0; k < kCloseBuckets; ++k) {
-    g->cstats.bucket_teams[k] = (uint64_t)n[k];
-    g->cstats.teams += (uint64_t)n[k];
+    g->cstats.bucket_teams[k] = (uint64_t)h.label_count[k];
+    g->cstats.teams += (uint64_t)h.label_count[k];
   }
-  g->cstats.bucket_teams[kWideBucket] += (uint64_t)n_over;   // handed from the warp kernels
+  g->cstats.bucket_teams[kWideBucket] += (uint64_t)n_over;   // handed from the other teams
   g->counted = true;
   g->have_cstats = true;
   if (counts) std::memcpy(counts, g->counts, sizeof(g->counts));

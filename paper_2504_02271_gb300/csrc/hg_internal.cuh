@@ -52,6 +52,14 @@ struct DevGraph {
   // [m_eoff[m], m_eoff[m+1]); nm == 0 for a single hypergraph
   const int32_t* m_eoff;
   int32_t nm;
+  // step two, set once the build is done (null before): per hyperedge x its start in e_idx
+  // (two words), |e_x| and its out-degree in one 16-byte record; osum[u] = sum over
+  // x in out(u) of |e_x| rounded up to a multiple of four, dsum[u] = the sum of their degrees
+  // (both at most 2^31 - 1); cand[u] = sum over its vertices of |E_y| - 1
+  const uint4* rec;
+  const int32_t* osum;
+  const int32_t* dsum;
+  const int64_t* cand;
 };
 
 // member owning hyperedge u (0 for a single hypergraph)
@@ -74,8 +82,12 @@ void note_launch(int n = 1);
 size_t scan_tmp_bytes(int64_t n);
 void scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, void* tmp, cudaStream_t s);
 void scan_i64_to_i64(const int64_t* in, int64_t* out, int64_t n, void* tmp, cudaStream_t s);
-// acc[0] += sum C(x,2), acc[1] = max x, acc[2] += sum x  over x in a[0..n)
-void reduce_deg_stats(const int32_t* a, int64_t n, unsigned long long* acc, cudaStream_t s);
+// acc[0] += sum C(x,2), acc[1] = max x, acc[2] += sum x over x in deg (dplus) [0..n), and
+// ds[i] = (deg[i], esize[i]) (rec[i] = (e_ptr[i] in two words, esize[i], dplus[i]))
+void launch_deg_stats(const int32_t* deg, const int32_t* esize, int64_t n,
+                      unsigned long long* acc, int2* ds, cudaStream_t s);
+void launch_out_stats(const int32_t* dplus, const int64_t* e_ptr, const int32_t* esize, int64_t n,
+                      unsigned long long* acc, uint4* rec, cudaStream_t s);
 
 // k_load.cu
 // One thread waits until *flag != 0, at most limit_ns of the global timer (and a bounded
@@ -144,10 +156,12 @@ void launch_cap_rows(const int64_t* cand, int32_t ne, int32_t* cap, cudaStream_t
 // Filter rows of the capacity layout (len[i] entries from src_ptr[i]) into an exact layout
 // (row i from dst_ptr[i]), order kept: keep 0 = j ranked above i in (deg, id), 1 = j > i,
 // 2 = all.  count_only: write the number kept to cnt[i] instead.
+// ds: (deg, |e|) of every hyperedge (keep 0 only); osum, dsum (keep 0, may be null): see
+// DevGraph.
 void launch_filter_rows(int keep, bool count_only, const int64_t* src_ptr, const int32_t* len,
-                        const Oriented& src, const int32_t* deg, int32_t ne, int packed,
+                        const Oriented& src, const int2* ds, int32_t ne, int packed,
                         const int64_t* dst_ptr, const Oriented& dst, int32_t* cnt,
-                        cudaStream_t s);
+                        int32_t* osum, int32_t* dsum, cudaStream_t s);
 
 // hg_api.cu: allocations of the calling thread skip the caller-installed hooks
 void alloc_bypass_hooks(bool on);
@@ -208,40 +222,108 @@ void launch_gather_rows(const int64_t* e_ptr, const int32_t* e_idx, const int32_
                         const int64_t* sub_ptr, int32_t* sub_idx, cudaStream_t s);
 size_t wedge_heavy_scratch_bytes(int64_t heavy_max_cand, int nsm);
 
-// k_close.cu
-// close team shapes: warp teams (out-degree <= 64, 128, 256), block teams with shared
-// tables (<= 1024, <= 2048, and <= kBlockMaxPacked or kBlockMaxUnpacked by the row
-// layout), block teams with global scratch (|e_u| > 32 with out-degree <= kWideLargeMin,
-// and teams handed over), cluster teams with global scratch (the rest)
+// Step two.  Shapes a caller sees (hg_close_stats): by out-degree and |e_u|, see
+// TeamRule::label.  Lists of owners the kernels take: one per kernel shape.
 constexpr int kCloseBuckets = 8;
 constexpr int kWideBucket = 6;
 constexpr int kClusterBucket = 7;
 constexpr int kWideLargeMin = 4096;
-constexpr int kBlockMaxPacked = 6144;     // 4-byte queue entries leave room for 6,144 indices
+constexpr int kWarpMaskBits = 32;         // one-word masks of the warp teams
+constexpr int kBlockMaxPacked = 6144;
 constexpr int kBlockMaxUnpacked = 4096;
-struct CloseBuckets {
-  int32_t* lists[kCloseBuckets];
-  int32_t* count;     // [kCloseBuckets]
+
+struct TeamRule {
+  int all_wide;    // every owner to the global-table blocks
+  int warp_max;    // largest out-degree labelled a warp team (64, 128 or 256)
+  int block_max;   // largest out-degree labelled a block team
+  // shape of an owner with out-degree d and sz vertices (-1: it closes nothing)
+  __host__ __device__ int label(int32_t d, int32_t sz) const {
+    if (d < 2) return -1;
+    if (all_wide) return kWideBucket;
+    if (sz <= kWarpMaskBits && d <= warp_max) return d <= 64 ? 0 : (d <= 128 ? 1 : 2);
+    if (sz <= kWarpMaskBits && d <= 1024) return 3;
+    if (sz <= kWarpMaskBits && d <= 2048) return 4;
+    if (sz <= kWarpMaskBits && d <= block_max) return 5;
+    return d > kWideLargeMin ? kClusterBucket : kWideBucket;
+  }
 };
-// all_block: send every hyperedge to the global-table kernel (bucket 6)
-// warp_max: the largest out-degree a warp team takes (64, 128 or 256); larger out-degrees
-// (and |e_u| > 32) go to block teams
+
+// Lists: warp teams that walk the out-lists (labels 0-2), the bit-row classes, global-table
+// blocks, global-table clusters, and the owners no other list takes or that a team handed
+// over.
+constexpr int kListBits = 3;
+constexpr int kBitClasses = 6;
+constexpr int kListWide = kListBits + kBitClasses;
+constexpr int kListCluster = kListWide + 1;
+constexpr int kListOver = kListCluster + 1;
+constexpr int kLists = kListOver + 1;
+constexpr int kWalkRatio0 = 8, kWalkRatio3 = 40, kWalkRatio4 = 80;   // see list_of in k_close.cu
+constexpr int kBitMaxOut = 8192;             // bit rows: out-degree, column-list entries
+constexpr int kBitMaxEntries = 1 << 22;
+constexpr int kBitDirectVertices = 32768;    // direct vertex map up to this many vertices
+
+constexpr int kBitSmem = 232448 - 2048;      // dynamic shared memory a block may take
+constexpr int kBitPlanes = 16;               // digits of a shared count (<= 65,535)
+constexpr int kBitLargeSlots = 14;           // log2 slots of the last class's hash dictionary
+
+// Shared memory of the last class before its columns: digits and flags, e_u's columns
+// twice, the rows, and the vertex dictionary.
+__host__ __device__ inline int64_t bit_large_bytes(int64_t du, int64_t szu, int64_t nv) {
+  const int64_t W = (du + 31) / 32;
+  return 4 * (kBitPlanes + 1) * W + 8 * szu * W + 23 * du +
+         (nv <= kBitDirectVertices ? 8 * ((nv + 31) / 32) + 2 * nv : 6ll << kBitLargeSlots) + 256;
+}
+
+// Smallest bit-row class that holds an owner (k_bits.cu, kShapes), -1 for none.  osum: see
+// DevGraph (an upper bound of the column list, and with szu of the dictionary's keys).
+__host__ __device__ inline int bit_class_of(int64_t du, int64_t szu, int64_t osum, int64_t nv) {
+  const int64_t mw = szu * ((du + 31) / 32), e = osum + szu;
+  if (szu <= kWarpMaskBits) {
+    if (du <= 64 && e <= 512 && mw <= 128) return 0;
+    if (du <= 128 && e <= 1024 && mw <= 256) return 1;
+    if (du <= 256 && e <= 2048 && mw <= 512) return 2;
+    if (du <= 512 && e <= 4096 && mw <= 1024) return 3;
+    if (du <= 1024 && e <= 8192 && mw <= 2048) return 4;
+  }
+  // (32 KB of columns at least)
+  if (du <= kBitMaxOut && e <= kBitMaxEntries && szu <= 4096 &&
+      bit_large_bytes(du, szu, nv) <= kBitSmem - 32768)
+    return 5;
+  return -1;
+}
+
+// k_close.cu
+struct CloseLists {
+  int32_t* lists[kLists];
+  int32_t* count;         // [kLists]
+  int32_t* labels;        // [kCloseBuckets] owners per label
+  unsigned long long* maxima;   // largest [0] out-degree, [1] |e_u| of the wide and cluster
+                                // lists, [2], [3] of all, [4] osum, [5] out-degree of the
+                                // last bit class
+};
 // sel: NULL, or one byte per hyperedge; then only the hyperedges u with sel[u] != 0
 // get a team (the hyper-triangles they own).
-// block_max: largest out-degree of the shared-table block teams (kBlockMaxPacked or
-// kBlockMaxUnpacked, by the row layout).
-void launch_bucket_close(const DevGraph& g, const Oriented& o, CloseBuckets b,
-                         unsigned long long* wide_max, bool all_block, int warp_max,
-                         int block_max, const uint8_t* sel, cudaStream_t s);
-// n: list length (host copy); n_p: the same on the device; counter: zeroed fetch counter;
-// work[0] += probes (entries of out(v) streamed), work[1] += E_y entries scanned for masks;
-// warp kernels append hyperedges their tables cannot hold (every hyperedge when
-// handover is set) to overflow[*n_overflow++]
-void launch_close(int bucket, const DevGraph& g, const Oriented& o, int packed,
+void launch_bucket_close(const DevGraph& g, const Oriented& o, CloseLists b, const TeamRule& rule,
+                         const uint8_t* sel, cudaStream_t s);
+// list: 0, 1, 2 (warp teams by label), kListWide, kListCluster or kListOver; n: its length
+// (host copy); n_p: the same on the device; counter: zeroed fetch counter; work[0] += probes,
+// work[1] += E_y entries, work[2] += out-entries (hg_close_stats); the warp teams append
+// owners their tables cannot hold (every one when handover is set) to
+// overflow[*n_overflow++]
+cudaError_t launch_close(int list_id, const DevGraph& g, const Oriented& o, int packed,
                   const int32_t* list, int32_t n, const int32_t* n_p, int64_t wide_cap,
                   int64_t wide_words, int64_t wide_dmax, void* scratch, unsigned long long* hist,
                   unsigned long long* work, int32_t* counter, int32_t* overflow,
                   int32_t* n_overflow, int handover, cudaStream_t s, int nsm);
+// k_bits.cu: the owners of bit-row class c.  work: [kCloseBuckets][3] as above, by label.
+// The last class keeps `slice` bytes of scratch per block, at most blocks_max blocks.
+int64_t bits_slice_bytes(int64_t dmax, int64_t imax);
+cudaError_t launch_close_bits(int c, const DevGraph& g, const Oriented& o, int packed,
+                       const int32_t* list, int32_t n, const int32_t* n_p, void* scratch,
+                       int64_t slice, int64_t dmax, int blocks_max, unsigned long long* hist,
+                       unsigned long long* work, const TeamRule& rule, int32_t* counter,
+                       int32_t* overflow, int32_t* n_overflow, int handover, cudaStream_t s,
+                       int nsm);
 size_t close_wide_scratch_bytes(int64_t cap, int64_t words, int64_t dmax, int nsm);
 
 }  // namespace hg

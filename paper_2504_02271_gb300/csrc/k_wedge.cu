@@ -375,31 +375,52 @@ __device__ __forceinline__ void get_row_entry(const Oriented& o, int64_t at, uin
 // kept, into cnt[i]; otherwise the rows, and the number kept into cnt[i] when cnt is set.
 template <int KEEP, bool PACKED, bool COUNT>
 __global__ void k_filter_rows(const int64_t* __restrict__ src_ptr, const int32_t* __restrict__ len,
-                              Oriented src, const int32_t* __restrict__ deg, int32_t ne,
+                              Oriented src, const int2* __restrict__ ds, int32_t ne,
                               const int64_t* __restrict__ dst_ptr, Oriented dst,
-                              int32_t* __restrict__ cnt) {
+                              int32_t* __restrict__ cnt, int32_t* __restrict__ osum,
+                              int32_t* __restrict__ dsum) {
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   for (int32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < ne; i += warps) {
     const int64_t b = src_ptr[i];
     const int32_t n = len[i];
-    const int32_t di = KEEP == 0 ? deg[i] : 0;
+    const int32_t di = KEEP == 0 ? ds[i].x : 0;
     const int64_t out = COUNT ? 0 : dst_ptr[i];
     int32_t kept = 0;
+    unsigned long long sum = 0, dsm = 0;
     for (int32_t t0 = 0; t0 < n; t0 += 32) {
       const int32_t t = t0 + lane;
       bool keep = false;
       uint32_t j = 0, om = 0;
       if (t < n) {
         get_row_entry<PACKED>(src, b + t, j, om);
-        keep = KEEP == 0 ? ranked_above(di, i, deg[j], (int32_t)j)
-                         : (KEEP == 1 ? (int32_t)j > i : true);
+        if (KEEP == 0) {
+          const int2 dj = ds[j];
+          keep = ranked_above(di, i, dj.x, (int32_t)j);
+          if (keep) {
+            sum += (unsigned long long)((dj.y + 3) & ~3);
+            dsm += (unsigned long long)dj.x;
+          }
+        } else {
+          keep = KEEP == 1 ? (int32_t)j > i : true;
+        }
       }
       const unsigned bal = __ballot_sync(kFull, keep);
       if (!COUNT && keep) put_entry<PACKED>(dst, out + kept + __popc(bal & ((1u << lane) - 1u)), j, om);
       kept += __popc(bal);
     }
     if (lane == 0 && cnt) cnt[i] = kept;
+    if (KEEP == 0 && !COUNT) {
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) {
+        sum += __shfl_down_sync(kFull, sum, d);
+        dsm += __shfl_down_sync(kFull, dsm, d);
+      }
+      if (lane == 0 && osum) {
+        osum[i] = sum < 0x7fffffffull ? (int32_t)sum : 0x7fffffff;
+        dsum[i] = dsm < 0x7fffffffull ? (int32_t)dsm : 0x7fffffff;
+      }
+    }
   }
 }
 
@@ -484,15 +505,18 @@ int grid_rows(int64_t rows, int per_block) {
 
 template <int KEEP, bool PACKED>
 void launch_filter_t(bool count_only, const int64_t* src_ptr, const int32_t* len,
-                     const Oriented& src, const int32_t* deg, int32_t ne, const int64_t* dst_ptr,
-                     const Oriented& dst, int32_t* cnt, cudaStream_t s) {
+                     const Oriented& src, const int2* ds, int32_t ne, const int64_t* dst_ptr,
+                     const Oriented& dst, int32_t* cnt, int32_t* osum, int32_t* dsum,
+                     cudaStream_t s) {
   note_launch();
   if (count_only)
-    k_filter_rows<KEEP, PACKED, true><<<grid_rows(ne, 8), 256, 0, s>>>(src_ptr, len, src, deg, ne,
-                                                                        dst_ptr, dst, cnt);
+    k_filter_rows<KEEP, PACKED, true><<<grid_rows(ne, 8), 256, 0, s>>>(src_ptr, len, src, ds, ne,
+                                                                        dst_ptr, dst, cnt, osum,
+                                                                        dsum);
   else
-    k_filter_rows<KEEP, PACKED, false><<<grid_rows(ne, 8), 256, 0, s>>>(src_ptr, len, src, deg,
-                                                                         ne, dst_ptr, dst, cnt);
+    k_filter_rows<KEEP, PACKED, false><<<grid_rows(ne, 8), 256, 0, s>>>(src_ptr, len, src, ds,
+                                                                         ne, dst_ptr, dst, cnt,
+                                                                         osum, dsum);
 }
 
 }  // namespace
@@ -536,15 +560,17 @@ void launch_cap_rows(const int64_t* cand, int32_t ne, int32_t* cap, cudaStream_t
 }
 
 void launch_filter_rows(int keep, bool count_only, const int64_t* src_ptr, const int32_t* len,
-                        const Oriented& src, const int32_t* deg, int32_t ne, int packed,
+                        const Oriented& src, const int2* ds, int32_t ne, int packed,
                         const int64_t* dst_ptr, const Oriented& dst, int32_t* cnt,
-                        cudaStream_t s) {
+                        int32_t* osum, int32_t* dsum, cudaStream_t s) {
   if (ne == 0) return;
 #define HG_FILTER(K)                                                                        \
   if (packed)                                                                              \
-    launch_filter_t<K, true>(count_only, src_ptr, len, src, deg, ne, dst_ptr, dst, cnt, s); \
+    launch_filter_t<K, true>(count_only, src_ptr, len, src, ds, ne, dst_ptr, dst, cnt, osum, \
+                             dsum, s);                                                     \
   else                                                                                     \
-    launch_filter_t<K, false>(count_only, src_ptr, len, src, deg, ne, dst_ptr, dst, cnt, s);
+    launch_filter_t<K, false>(count_only, src_ptr, len, src, ds, ne, dst_ptr, dst, cnt, osum, \
+                              dsum, s);
   if (keep == 0) {
     HG_FILTER(0)
   } else if (keep == 1) {
