@@ -132,6 +132,7 @@ struct hg_graph {
   int32_t nm = 0;
   int32_t* m_eoff = nullptr;
   int32_t* m_voff = nullptr;
+  int32_t max_member_nv = 0;              // most vertices of a member
   int32_t* wcr = nullptr;                 // per-row inclusion wedges (build)
   unsigned long long* mstats = nullptr;   // [nm][4]: sum deg, sum C(deg,2), W_c, max deg
   unsigned long long* mhist = nullptr;    // [nm][128] labelled region-mask bins (count)
@@ -503,6 +504,8 @@ hg_status load_impl(hg_graph* g, const int64_t* edge_ptr, const int32_t* edge_vt
                             cudaMemcpyHostToDevice, s));
     HG_CUDA(cudaMemcpyAsync(g->m_voff, wave->voff, sizeof(int32_t) * ((size_t)g->nm + 1),
                             cudaMemcpyHostToDevice, s));
+    for (int32_t m = 0; m < g->nm; ++m)
+      g->max_member_nv = std::max(g->max_member_nv, wave->voff[m + 1] - wave->voff[m]);
     if (wave->m_eptr) {
       int64_t* noff = alloc_t<int64_t>(g, g->load_blocks, (int64_t)g->nm + 1);
       if (!noff) return HG_ERR_OOM;
@@ -564,8 +567,12 @@ hg_status dense_impl(hg_graph* g, const hg_tuning* opt, DenseInfo* dn) {
     t = k;
   }
   if (above == 0 || (!forced && above < kDenseMinRows)) return HG_OK;
-  const int64_t rows_pad = dense_round_rows(above), k_pad = dense_round_k(g->nv);
-  if (rows_pad * (k_pad + 2 * rows_pad) > kDenseMaxBytes) return HG_OK;   // stays on the hash path
+  const int64_t rows_pad = dense_round_rows(above);
+  if (rows_pad * (dense_round_k(g->nv) + 2 * rows_pad) > kDenseMaxBytes)
+    return HG_OK;   // stays on the hash path
+  // a batch: member-local columns, and only the tiles inside members (see k_dense.cu)
+  const bool batch = g->nm > 0;
+  const int64_t k_pad = dense_round_k(batch ? g->max_member_nv : g->nv);
   int32_t* heavy_idx = alloc_t<int32_t>(g, g->build_blocks, g->ne);
   int32_t* ids = alloc_t<int32_t>(g, g->build_blocks, above);
   uint8_t* a = alloc_t<uint8_t>(g, g->build_blocks, rows_pad * k_pad);
@@ -574,10 +581,31 @@ hg_status dense_impl(hg_graph* g, const hg_tuning* opt, DenseInfo* dn) {
   int32_t* count = g->small->counters + 8;
   HG_CUDA(cudaMemsetAsync(count, 0, sizeof(int32_t), s));
   HG_CUDA(cudaMemsetAsync(a, 0, (size_t)(rows_pad * k_pad), s));
-  launch_pick_heavy(g->esize, g->ne, t, kDenseMaxOmega, (int32_t)above, heavy_idx, ids, count, s);
-  launch_fill_dense(g->e_ptr, g->e_idx, ids, (int32_t)above, a, k_pad, s);
+  const DevGraph d = dev_graph(g);
+  int4* list = nullptr;
+  int32_t* list_n = nullptr;
+  int2* hrange = nullptr;
+  if (batch) {
+    int32_t* flag = nullptr;
+    int64_t* rank = nullptr;
+    Carver c;
+    c.want(flag, g->ne);
+    c.want(rank, (int64_t)g->ne + 1);
+    c.want(hrange, g->nm);
+    c.want(list, dense_tiles(rows_pad));
+    c.want(list_n, 1);
+    if (!c.get(g, g->build_blocks)) return HG_ERR_OOM;
+    HG_CUDA(cudaMemsetAsync(hrange, 0, sizeof(int2) * (size_t)g->nm, s));
+    launch_heavy_flags(g->esize, g->ne, t, kDenseMaxOmega, flag, s);
+    scan_i32_to_i64(flag, rank, g->ne, g->scan_tmp, s);
+    launch_heavy_place(d, flag, rank, (int32_t)above, heavy_idx, ids, count, hrange, s);
+    launch_tile_list(d, ids, (int32_t)above, g->m_voff, rows_pad, list, list_n, s);
+  } else {
+    launch_pick_heavy(g->esize, g->ne, t, kDenseMaxOmega, (int32_t)above, heavy_idx, ids, count, s);
+  }
+  launch_fill_dense(d, ids, (int32_t)above, a, k_pad, batch ? g->m_voff : nullptr, s);
   t_begin(g, "dense_omega");
-  HG_CUDA(launch_dense_omega(a, above, rows_pad, k_pad, omega, &g->small->err, s));
+  HG_CUDA(launch_dense_omega(a, above, rows_pad, k_pad, list, list_n, omega, &g->small->err, s));
   t_end(g);
   Small hs;
   HG_TRY(sync_small(g, &hs));
@@ -587,6 +615,7 @@ hg_status dense_impl(hg_graph* g, const hg_tuning* opt, DenseInfo* dn) {
   dn->omega = omega;
   dn->ld = rows_pad;
   dn->nh = (int32_t)above;
+  dn->hrange = hrange;
   return HG_OK;
 }
 
@@ -745,6 +774,7 @@ hg_status build_impl(hg_graph* g, const hg_tuning* opt, hg_wedge_stats* out) {
   t_end(g);
   if (g->nm > 0) {
     g->h_mstats.assign(4 * (size_t)g->nm, 0);
+    HG_CUDA(cudaMemsetAsync(g->mstats, 0, sizeof(unsigned long long) * g->h_mstats.size(), s));
     launch_member_stats(d, g->deg, g->wcr, g->mstats, s);
     HG_CUDA(cudaMemcpyAsync(g->h_mstats.data(), g->mstats, sizeof(unsigned long long) * g->h_mstats.size(),
                             cudaMemcpyDeviceToHost, s));

@@ -109,6 +109,7 @@ struct DenseInfo {
   const uint16_t* omega;      // [rows_pad x rows_pad] omega of heavy pairs
   int64_t ld;                 // row stride of omega
   int32_t nh;
+  const int2* hrange;         // a batch: [first, end) heavy positions of every member; else null
 };
 size_t dense_smem_bytes();
 int64_t dense_round_rows(int64_t n);
@@ -121,10 +122,24 @@ void launch_pick_heavy(const int32_t* esize, int32_t ne, int32_t min_size, int32
                        cudaStream_t s);
 // omega values the tile kernel writes exactly (uint16 output)
 constexpr int32_t kDenseMaxOmega = 65535;
-void launch_fill_dense(const int64_t* e_ptr, const int32_t* e_idx, const int32_t* ids, int32_t nh,
-                       uint8_t* a, int64_t lda, cudaStream_t s);
+// the same for a batch, member by member: flag[i], then (rank = prefix sums of flag) places and
+// every member's range of heavy positions (hrange cleared before)
+void launch_heavy_flags(const int32_t* esize, int32_t ne, int32_t min_size, int32_t max_size,
+                        int32_t* flag, cudaStream_t s);
+void launch_heavy_place(const DevGraph& g, const int32_t* flag, const int64_t* rank, int32_t cap,
+                        int32_t* heavy_idx, int32_t* ids, int32_t* count, int2* hrange,
+                        cudaStream_t s);
+// a batch's tiles with work (at most dense_tiles(rows_pad)) and their number
+int64_t dense_tiles(int64_t rows_pad);
+void launch_tile_list(const DevGraph& g, const int32_t* ids, int32_t nh, const int32_t* voff,
+                      int64_t rows_pad, int4* list, int32_t* list_n, cudaStream_t s);
+// voff: member vertex offsets (columns are member-local then), or null
+void launch_fill_dense(const DevGraph& g, const int32_t* ids, int32_t nh, uint8_t* a, int64_t lda,
+                       const int32_t* voff, cudaStream_t s);
+// list, list_n: launch_tile_list's, or null (every tile, every step of K)
 cudaError_t launch_dense_omega(const uint8_t* a, int64_t rows, int64_t rows_pad, int64_t k_pad,
-                               uint16_t* omega, int* err, cudaStream_t s);
+                               const int4* list, const int32_t* list_n, uint16_t* omega, int* err,
+                               cudaStream_t s);
 
 // k_wedge.cu
 struct WedgeBuckets {

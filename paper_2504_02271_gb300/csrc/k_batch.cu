@@ -51,36 +51,45 @@ __global__ void k_localize(DevGraph g, const int32_t* __restrict__ m_voff, int32
   }
 }
 
-// One warp per member: out[4m..4m+3] = sum deg (= 2 W_m), sum C(deg, 2), inclusion
-// wedges W_c, max deg.
+// out[4m..4m+3] += sum deg (= 2 W_m), sum C(deg, 2), inclusion wedges W_c, max deg of member
+// m (cleared before).  One warp per kStatRows rows, whatever their members: with one warp per
+// member the largest member's rows took 2.0 ms of a 64-member batch.
+constexpr int kStatRows = 512;
+
 __global__ void k_member_stats(DevGraph g, const int32_t* __restrict__ deg,
                                const int32_t* __restrict__ wcr,
                                unsigned long long* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
-  for (int32_t m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; m < g.nm; m += warps) {
-    const int32_t b = g.m_eoff[m], e = g.m_eoff[m + 1];
-    unsigned long long sd = 0, sc2 = 0, swc = 0, mx = 0;
-    for (int32_t i = b + lane; i < e; i += 32) {
-      const unsigned long long d = (unsigned long long)deg[i];
-      sd += d;
-      sc2 += d * (d - (d > 0)) / 2;
-      swc += (unsigned long long)wcr[i];
-      mx = d > mx ? d : mx;
-    }
+  for (int64_t r0 = (int64_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kStatRows; r0 < g.ne;
+       r0 += (int64_t)warps * kStatRows) {
+    const int32_t r1 = (int32_t)(r0 + kStatRows < g.ne ? r0 + kStatRows : g.ne);
+    for (int32_t b = (int32_t)r0; b < r1;) {   // the rows of one member at a time
+      const int32_t m = member_of(g, b);
+      const int32_t e = g.m_eoff[m + 1] < r1 ? g.m_eoff[m + 1] : r1;
+      unsigned long long sd = 0, sc2 = 0, swc = 0, mx = 0;
+      for (int32_t i = b + lane; i < e; i += 32) {
+        const unsigned long long d = (unsigned long long)deg[i];
+        sd += d;
+        sc2 += d * (d - (d > 0)) / 2;
+        swc += (unsigned long long)wcr[i];
+        mx = d > mx ? d : mx;
+      }
 #pragma unroll
-    for (int k = 16; k > 0; k >>= 1) {
-      sd += __shfl_down_sync(kFull, sd, k);
-      sc2 += __shfl_down_sync(kFull, sc2, k);
-      swc += __shfl_down_sync(kFull, swc, k);
-      const unsigned long long o = __shfl_down_sync(kFull, mx, k);
-      mx = o > mx ? o : mx;
-    }
-    if (lane == 0) {
-      out[4 * (size_t)m + 0] = sd;
-      out[4 * (size_t)m + 1] = sc2;
-      out[4 * (size_t)m + 2] = swc;
-      out[4 * (size_t)m + 3] = mx;
+      for (int k = 16; k > 0; k >>= 1) {
+        sd += __shfl_down_sync(kFull, sd, k);
+        sc2 += __shfl_down_sync(kFull, sc2, k);
+        swc += __shfl_down_sync(kFull, swc, k);
+        const unsigned long long o = __shfl_down_sync(kFull, mx, k);
+        mx = o > mx ? o : mx;
+      }
+      if (lane == 0) {
+        atomicAdd(&out[4 * (size_t)m + 0], sd);
+        atomicAdd(&out[4 * (size_t)m + 1], sc2);
+        atomicAdd(&out[4 * (size_t)m + 2], swc);
+        atomicMax(&out[4 * (size_t)m + 3], mx);
+      }
+      b = e;
     }
   }
 }
@@ -117,7 +126,7 @@ void launch_member_stats(const DevGraph& g, const int32_t* deg, const int32_t* w
                          unsigned long long* out, cudaStream_t s) {
   if (g.nm == 0) return;
   note_launch();
-  k_member_stats<<<grid_of(g.nm, 8), 256, 0, s>>>(g, deg, wcr, out);
+  k_member_stats<<<grid_of(g.ne, 8 * kStatRows), 256, 0, s>>>(g, deg, wcr, out);
 }
 
 }  // namespace hg

@@ -84,6 +84,11 @@ __device__ __forceinline__ void ht_add(typename GatherSlot<PACKED>::T* T, int ca
 
 // Row i of a heavy hyperedge: its heavy neighbours come from the dense tiles, so the
 // gather skips them; light rows (and a graph without a dense path) gather everything.
+// heavy positions row i's tiles were multiplied for: its member's in a batch, else all
+__device__ __forceinline__ int2 heavy_range(const DevGraph& g, const DenseInfo& dn, int32_t i) {
+  return dn.hrange ? dn.hrange[member_of(g, i)] : make_int2(0, dn.nh);
+}
+
 __device__ __forceinline__ bool gather_pair(const DenseInfo& dn, int32_t hi, int32_t j) {
   return hi < 0 || dn.heavy_idx[j] < 0;
 }
@@ -179,7 +184,8 @@ __global__ void __launch_bounds__(kLightWarps * 32, HG_LIGHT_MIN_BLOCKS)
       }
     }
     if (hi >= 0) {
-      for (int32_t h = lane; h < dn.nh; h += 32) {
+      const int2 hr = heavy_range(g, dn, i);
+      for (int32_t h = hr.x + lane; h < hr.y; h += 32) {
         const uint32_t om = dn.omega[(int64_t)hi * dn.ld + h];
         if (om && h != hi) ht_add<PACKED>(T, cl, (uint32_t)dn.ids[h], om);
       }
@@ -302,7 +308,8 @@ __global__ void __launch_bounds__(kBlockThreads)
       __syncthreads();   // the next chunk rewrites the ranges
     }
     if (hi >= 0) {
-      for (int32_t h = threadIdx.x; h < dn.nh; h += kBlockThreads) {
+      const int2 hr = heavy_range(g, dn, i);
+      for (int32_t h = hr.x + (int)threadIdx.x; h < hr.y; h += kBlockThreads) {
         const uint32_t om = dn.omega[(int64_t)hi * dn.ld + h];
         if (om && h != hi) ht_add<PACKED>(T, cl, (uint32_t)dn.ids[h], om);
       }
