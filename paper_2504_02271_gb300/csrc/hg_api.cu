@@ -829,7 +829,8 @@ hg_status upper_impl(hg_graph* g) {
                      g->up_ptr, g->up, nullptr, nullptr, nullptr, s);
   t_end(g);
   t_begin(g, "upper_sort");
-  HG_CUDA(launch_sort_upper(g->up_ptr, g->ne, g->up, g->packed, &g->small->err, s, g->nsm));
+  HG_CUDA(launch_sort_upper(g->up_ptr, g->ne, g->up, g->packed, g->stats.max_deg, &g->small->err,
+                            s, g->nsm));
   t_end(g);
   g->up_index = alloc_t<int32_t>(g, g->sample_blocks,
                                  row_index_buckets(g->stats.W, row_index_shift(g->stats.W, g->ne)) + 1);
@@ -898,7 +899,8 @@ hg_status adv_impl(hg_graph* g) {
                      g->deg_ptr, g->full, nullptr, nullptr, nullptr, s);
   t_end(g);
   t_begin(g, "full_sort");
-  HG_CUDA(launch_sort_upper(g->deg_ptr, g->ne, g->full, g->packed, &g->small->err, s, g->nsm));
+  HG_CUDA(launch_sort_upper(g->deg_ptr, g->ne, g->full, g->packed, g->stats.max_deg,
+                            &g->small->err, s, g->nsm));
   t_end(g);
   Small h;
   HG_TRY(sync_small(g, &h));

@@ -193,8 +193,9 @@ void launch_member_stats(const DevGraph& g, const int32_t* deg, const int32_t* w
 // k_sample.cu
 int sample_sort_max_log2();
 void sample_set_lut(const uint8_t lut[128], cudaStream_t s);
+// max_len: an upper bound of the row lengths
 cudaError_t launch_sort_upper(const int64_t* up_ptr, int32_t ne, const Oriented& up, int packed,
-                              int* err, cudaStream_t s, int nsm);
+                              uint64_t max_len, int* err, cudaStream_t s, int nsm);
 // Bucket index of a row-pointer array of `entries` entries over ne rows (sampler row
 // searches): row_index_buckets(entries, row_index_shift(entries, ne)) + 1 int32.
 int row_index_shift(uint64_t entries, int32_t rows);

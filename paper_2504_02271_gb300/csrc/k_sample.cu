@@ -10,7 +10,9 @@
 // {i, j, k} whose smallest hyperwedge in O is (i, j); it is classified from its
 // seven Venn regions (g = |e_i cap e_j cap e_k| from the staged e_i cap e_j) and
 // counted.
+#include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "hg_internal.cuh"
 
@@ -39,61 +41,130 @@ __device__ __forceinline__ void philox4x32_10(uint32_t c[4], uint32_t k0, uint32
   }
 }
 
-// Sort each upper row in shared memory (bitonic network on 64-bit keys
-// j << 32 | omega, padded to a power of two).  Rows longer than max_len set err.
+// Rows of up to kWarpSort entries: one warp each, a bitonic network in the warp's shared
+// memory (keys as stored in the packed layout, j << 32 | omega otherwise; padded to a power
+// of two).  A block per row spent its time in barriers and held 128 KB for about 40 entries:
+// an estimate on half of 150,000 co-authorship hyperedges, 1.33 ms of it this sort, went from
+// 3.50 to 2.41 ms.
+constexpr int kWarpSort = 512;
+
+template <bool PACKED>
+__global__ void __launch_bounds__(kSampleWarps * 32)
+    k_sort_rows(const int64_t* __restrict__ up_ptr, int32_t ne, Oriented up) {
+  using Key = typename std::conditional<PACKED, uint32_t, unsigned long long>::type;
+  __shared__ Key keys[kSampleWarps][kWarpSort];
+  const int lane = threadIdx.x & 31;
+  Key* x = keys[threadIdx.x >> 5];
+  const int64_t warps = (int64_t)gridDim.x * kSampleWarps;
+  for (int64_t i = (int64_t)blockIdx.x * kSampleWarps + (threadIdx.x >> 5); i < ne; i += warps) {
+    const int64_t b = up_ptr[i], l = up_ptr[i + 1] - b;
+    if (l <= 1 || l > kWarpSort) continue;   // warp-uniform
+    const int len = (int)l;
+    int n = 32;
+    while (n < len) n <<= 1;
+    for (int t = lane; t < n; t += 32) {
+      Key key = ~(Key)0;
+      if (t < len)
+        key = PACKED ? (Key)up.packed[b + t]
+                     : (Key)((unsigned long long)(uint32_t)up.nbr[b + t] << 32 |
+                             (uint32_t)up.omega[b + t]);
+      x[t] = key;
+    }
+    __syncwarp();
+    for (int k = 2; k <= n; k <<= 1) {
+      for (int j = k >> 1; j > 0; j >>= 1) {
+        for (int t = lane; t < n / 2; t += 32) {
+          const int p = ((t & ~(j - 1)) << 1) | (t & (j - 1)), q = p | j;
+          const Key kp = x[p], kq = x[q];
+          if ((kp > kq) == ((p & k) == 0)) {
+            x[p] = kq;
+            x[q] = kp;
+          }
+        }
+        __syncwarp();
+      }
+    }
+    for (int t = lane; t < len; t += 32) {
+      const Key key = x[t];
+      if (PACKED) {
+        up.packed[b + t] = (uint32_t)key;
+      } else {
+        up.nbr[b + t] = (int32_t)((unsigned long long)key >> 32);
+        up.omega[b + t] = (int32_t)((unsigned long long)key & 0xffffffffu);
+      }
+    }
+    __syncwarp();
+  }
+}
+
+// Longer rows: one block each (bitonic network on 64-bit keys j << 32 | omega, padded to a
+// power of two).  Rows longer than max_len set err.  A block looks through kSortThreads
+// rows at once for those that are its own.
 __global__ void __launch_bounds__(kSortThreads)
     k_sort_upper(const int64_t* __restrict__ up_ptr, int32_t ne, Oriented up, int packed,
                  int max_len_log2, int* __restrict__ err) {
   extern __shared__ unsigned long long keys[];
-  for (int32_t i = blockIdx.x; i < ne; i += gridDim.x) {
-    const int64_t b = up_ptr[i];
-    const int32_t len = (int32_t)(up_ptr[i + 1] - b);
-    if (len <= 1) continue;
-    if (len > (1 << max_len_log2)) {
-      if (threadIdx.x == 0) dev_fail(err, DE_LIMIT);
-      continue;
-    }
-    int n = 1;
-    while (n < len) n <<= 1;
-    for (int t = threadIdx.x; t < n; t += kSortThreads) {
-      unsigned long long key = ~0ull;
-      if (t < len) {
-        if (packed) {
-          const uint32_t x = up.packed[b + t];
-          key = ((unsigned long long)(x >> 8) << 32) | (x & 0xffu);
-        } else {
-          key = ((unsigned long long)(uint32_t)up.nbr[b + t] << 32) | (uint32_t)up.omega[b + t];
-        }
-      }
-      keys[t] = key;
-    }
+  __shared__ int32_t s_row[kSortThreads], s_rows;
+  for (int64_t r0 = (int64_t)blockIdx.x * kSortThreads; r0 < ne;
+       r0 += (int64_t)gridDim.x * kSortThreads) {
+    if (threadIdx.x == 0) s_rows = 0;
     __syncthreads();
-    for (int k = 2; k <= n; k <<= 1) {
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        for (int t = threadIdx.x; t < n; t += kSortThreads) {
-          const int p = t ^ j;
-          if (p > t) {
-            const unsigned long long a = keys[t], c = keys[p];
-            const bool up_dir = (t & k) == 0;
-            if ((a > c) == up_dir) {
-              keys[t] = c;
-              keys[p] = a;
-            }
+    const int64_t mine = r0 + threadIdx.x;
+    if (mine < ne && up_ptr[mine + 1] - up_ptr[mine] > kWarpSort)
+      s_row[atomicAdd(&s_rows, 1)] = (int32_t)mine;
+    __syncthreads();
+    for (int rr = 0; rr < s_rows; ++rr) {
+      const int32_t i = s_row[rr];
+      const int64_t b = up_ptr[i];
+      const int64_t len64 = up_ptr[i + 1] - b;
+      const int32_t len = (int32_t)len64;
+      if (len64 > (1 << max_len_log2)) {
+        if (threadIdx.x == 0) dev_fail(err, DE_LIMIT);
+        continue;
+      }
+      int n = 1;
+      while (n < len) n <<= 1;
+      for (int t = threadIdx.x; t < n; t += kSortThreads) {
+        unsigned long long key = ~0ull;
+        if (t < len) {
+          if (packed) {
+            const uint32_t x = up.packed[b + t];
+            key = ((unsigned long long)(x >> 8) << 32) | (x & 0xffu);
+          } else {
+            key = ((unsigned long long)(uint32_t)up.nbr[b + t] << 32) | (uint32_t)up.omega[b + t];
           }
         }
-        __syncthreads();
+        keys[t] = key;
       }
-    }
-    for (int t = threadIdx.x; t < len; t += kSortThreads) {
-      const unsigned long long key = keys[t];
-      if (packed) {
-        up.packed[b + t] = ((uint32_t)(key >> 32) << 8) | (uint32_t)(key & 0xffu);
-      } else {
-        up.nbr[b + t] = (int32_t)(key >> 32);
-        up.omega[b + t] = (int32_t)(key & 0xffffffffu);
+      __syncthreads();
+      for (int k = 2; k <= n; k <<= 1) {
+        for (int j = k >> 1; j > 0; j >>= 1) {
+          for (int t = threadIdx.x; t < n; t += kSortThreads) {
+            const int p = t ^ j;
+            if (p > t) {
+              const unsigned long long a = keys[t], c = keys[p];
+              const bool up_dir = (t & k) == 0;
+              if ((a > c) == up_dir) {
+                keys[t] = c;
+                keys[p] = a;
+              }
+            }
+          }
+          __syncthreads();
+        }
       }
+      for (int t = threadIdx.x; t < len; t += kSortThreads) {
+        const unsigned long long key = keys[t];
+        if (packed) {
+          up.packed[b + t] = ((uint32_t)(key >> 32) << 8) | (uint32_t)(key & 0xffu);
+        } else {
+          up.nbr[b + t] = (int32_t)(key >> 32);
+          up.omega[b + t] = (int32_t)(key & 0xffffffffu);
+        }
+      }
+      __syncthreads();
     }
-    __syncthreads();
+    __syncthreads();   // (the list is rewritten)
   }
 }
 
@@ -772,8 +843,16 @@ void sample_set_lut(const uint8_t lut[128], cudaStream_t s) {
 }
 
 cudaError_t launch_sort_upper(const int64_t* up_ptr, int32_t ne, const Oriented& up, int packed,
-                              int* err, cudaStream_t s, int nsm) {
+                              uint64_t max_len, int* err, cudaStream_t s, int nsm) {
   if (ne == 0) return cudaSuccess;
+  note_launch();
+  const int64_t blocks = std::min<int64_t>(((int64_t)ne + kSampleWarps - 1) / kSampleWarps,
+                                           (int64_t)nsm * 16);
+  if (packed)
+    k_sort_rows<true><<<(unsigned)blocks, kSampleWarps * 32, 0, s>>>(up_ptr, ne, up);
+  else
+    k_sort_rows<false><<<(unsigned)blocks, kSampleWarps * 32, 0, s>>>(up_ptr, ne, up);
+  if (max_len <= (uint64_t)kWarpSort) return cudaGetLastError();
   const int smem = (int)(sizeof(unsigned long long) << kSortMaxLog2);
   cudaError_t e = cudaFuncSetAttribute(k_sort_upper, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        smem);
