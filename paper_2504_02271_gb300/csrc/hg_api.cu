@@ -1155,7 +1155,7 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
   if (n[kListWide] + n[kListCluster] > 0 && !wide_scratch(h.close_max[0], h.close_max[1], &wide))
     return HG_ERR_OOM;
   const int64_t slice_dmax = ((int64_t)h.close_max[5] + 15) / 16 * 16;
-  const int64_t slice = bits_slice_bytes(slice_dmax, (int64_t)h.close_max[4]);
+  const int64_t slice = bits_slice_bytes(slice_dmax, (int64_t)h.close_max[4], g->nv);
   const int slice_blocks = std::min(n[kListBits + kBitClasses - 1], g->nsm);
   void* slices = nullptr;
   if (slice_blocks > 0) {

@@ -276,7 +276,13 @@ constexpr int kLists = kListOver + 1;
 constexpr int kWalkRatio0 = 8, kWalkRatio3 = 40, kWalkRatio4 = 80;   // see list_of in k_close.cu
 constexpr int kBitMaxOut = 8192;             // bit rows: out-degree, column-list entries
 constexpr int kBitMaxEntries = 1 << 22;
-constexpr int kBitDirectVertices = 32768;    // direct vertex map up to this many vertices
+// Direct vertex map up to kBitDirectVertices; its bit maps alone in shared memory up to
+// kBitMapVertices (at most 64 KB, less than the hash), its columns in global scratch.  The hash
+// holds 16,384 vertices and an owner with more goes to the global-table blocks: closure of a
+// tag shape of 200,000 hyperedges over 40,000 vertices 1.56 against 0.35 s, of 300,000 over
+// 100,000 3.79 against 0.52 (the block teams before: 1.08, 1.57).
+constexpr int kBitDirectVertices = 32768;
+constexpr int kBitMapVertices = 262144;
 
 constexpr int kBitSmem = 232448 - 2048;      // dynamic shared memory a block may take
 constexpr int kBitPlanes = 16;               // digits of a shared count (<= 65,535)
@@ -287,7 +293,13 @@ constexpr int kBitLargeSlots = 14;           // log2 slots of the last class's h
 __host__ __device__ inline int64_t bit_large_bytes(int64_t du, int64_t szu, int64_t nv) {
   const int64_t W = (du + 31) / 32;
   return 4 * (kBitPlanes + 1) * W + 8 * szu * W + 23 * du +
-         (nv <= kBitDirectVertices ? 8 * ((nv + 31) / 32) + 2 * nv : 6ll << kBitLargeSlots) + 256;
+         (nv <= kBitMapVertices ? 8 * ((nv + 31) / 32) + (nv <= kBitDirectVertices ? 2 * nv : 0)
+                                : 6ll << kBitLargeSlots) + 256;
+}
+
+// Global scratch of a block for the columns by vertex.
+__host__ __device__ inline int64_t bits_val_bytes(int64_t nv) {
+  return nv > kBitDirectVertices && nv <= kBitMapVertices ? (2 * nv + 255) / 256 * 256 : 0;
 }
 
 // Smallest bit-row class that holds an owner (k_bits.cu, kShapes), -1 for none.  osum: see
@@ -333,7 +345,7 @@ cudaError_t launch_close(int list_id, const DevGraph& g, const Oriented& o, int 
                   int32_t* n_overflow, int handover, cudaStream_t s, int nsm);
 // k_bits.cu: the owners of bit-row class c.  work: [kCloseBuckets][3] as above, by label.
 // The last class keeps `slice` bytes of scratch per block, at most blocks_max blocks.
-int64_t bits_slice_bytes(int64_t dmax, int64_t imax);
+int64_t bits_slice_bytes(int64_t dmax, int64_t imax, int64_t nv);
 cudaError_t launch_close_bits(int c, const DevGraph& g, const Oriented& o, int packed,
                        const int32_t* list, int32_t n, const int32_t* n_p, void* scratch,
                        int64_t slice, int64_t dmax, int blocks_max, unsigned long long* hist,

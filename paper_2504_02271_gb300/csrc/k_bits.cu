@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(NW * 32, MINB)
       for (int k = tid; k < (1 << lg) / 4; k += NT) kv[k] = make_uint4(~0u, ~0u, ~0u, ~0u);
     }
     if (tid == 0) {
-      tb.used = tb.full = tb.inc = tb.ncand = tb.most = 
+      tb.used = tb.full = tb.inc = tb.ncand = tb.most = 0;
       tb.probes = 0;
       tb.ncol = szu;
     }
@@ -684,7 +684,8 @@ __global__ void __launch_bounds__(NW * 32, MINB)
 // One block of 32 warps per SM.  The list does not fit beside the columns, so the
 // hyperedges of out(u) are read twice, one warp per hyperedge with the next one's vertices
 // in flight: once to find the shared vertices, once to write the column lists.  The vertex
-// dictionary is a direct map while |V| allows (DIRECT), else a hash.  Column lists stay in
+// dictionary is a direct map while |V| allows, its columns in shared memory up to
+// kBitDirectVertices and in scratch (L2) up to kBitMapVertices, else a hash.  Column lists stay in
 // shared memory when they fit behind the dictionary, else in the block's slice of global
 // scratch; the columns then take the dictionary's place.
 
@@ -727,7 +728,11 @@ __device__ __forceinline__ void for_each_row(const DevGraph& g, const uint4* src
   }
 }
 
-template <bool PACKED, bool DIRECT>
+// Where the vertex dictionary of a large team lives: a hash; bit maps and columns by vertex in
+// shared memory; or the bit maps there and the columns in the block's slice of scratch.
+enum { kDictHash, kDictDirect, kDictMaps };
+
+template <bool PACKED, int DICT>
 __global__ void __launch_bounds__(kLargeWarps * 32, 1)
     k_bits_large(DevGraph g, Oriented o, int slots_log2, const int32_t* __restrict__ list,
                  const int32_t* __restrict__ n_p, char* __restrict__ scratch, int64_t slice,
@@ -736,11 +741,14 @@ __global__ void __launch_bounds__(kLargeWarps * 32, 1)
                  int32_t* __restrict__ counter, int32_t* __restrict__ overflow,
                  int32_t* __restrict__ n_overflow, int handover) {
   constexpr int NW = kLargeWarps, NT = NW * 32, G = 8;
+  constexpr bool DIRECT = DICT != kDictHash;
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ TeamBlock tb;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, tid = threadIdx.x;
   uint4* gsrc = reinterpret_cast<uint4*>(scratch + slice * blockIdx.x);   // [dmax]
   uint16_t* gcsr = reinterpret_cast<uint16_t*>(gsrc + dmax);
+  uint16_t* gval = reinterpret_cast<uint16_t*>(scratch + slice * (blockIdx.x + 1) -
+                                               bits_val_bytes(g.nv));
   for (int k = tid; k < kBins; k += NT) tb.hist[k] = 0;
   for (int k = tid; k < kCloseBuckets * 3; k += NT) (&tb.work[0][0])[k] = 0;
   const int32_t n = *n_p;
@@ -792,7 +800,10 @@ __global__ void __launch_bounds__(kLargeWarps * 32, 1)
     dict.words = (g.nv + 31) / 32;
     const uint32_t key_bytes = DIRECT ? 8u * (uint32_t)dict.words : 4u << slots_log2;
     dict.key = reinterpret_cast<uint32_t*>(dyn + take(key_bytes));
-    dict.val = reinterpret_cast<uint16_t*>(dyn + take(DIRECT ? 2u * (uint32_t)g.nv : 2u << slots_log2));
+    dict.val = DICT == kDictMaps
+                   ? gval
+                   : reinterpret_cast<uint16_t*>(
+                         dyn + take(DIRECT ? 2u * (uint32_t)g.nv : 2u << slots_log2));
     // the hyperedges' places in e_idx: in X when they fit, else in global scratch
     const uint32_t src_at = take(16u * du);
     const bool src_in = at <= (uint32_t)kBitSmem;
@@ -854,7 +865,9 @@ __global__ void __launch_bounds__(kLargeWarps * 32, 1)
     if (!over) {
       // 2. shared vertices
       for_each_row<NW>(g, src, du, lane, w, [&](int, uint32_t, int32_t v) {
-        if (v >= 0) dict.touch((uint32_t)v, &tb.ncol, &tb.full);
+        // (once it is full, every further vertex would take all its probes for nothing)
+        if (v >= 0 && (DIRECT || !*(volatile int*)&tb.full))
+          dict.touch((uint32_t)v, &tb.ncol, &tb.full);
       });
       if (tid == 0) tb.next = next.u;
       __syncthreads();
@@ -1020,13 +1033,13 @@ void launch_small(const DevGraph& g, const Oriented& o, const int32_t* list, int
                                             overflow, n_overflow, handover);
 }
 
-template <bool PACKED, bool DIRECT>
+template <bool PACKED, int DICT>
 void launch_large(const DevGraph& g, const Oriented& o, const int32_t* list, int32_t n,
                   const int32_t* n_p, void* scratch, int64_t slice, int64_t dmax, int blocks,
                   unsigned long long* hist, unsigned long long* work, const TeamRule& rule,
                   int32_t* counter, int32_t* overflow, int32_t* n_overflow, int handover,
                   cudaStream_t s) {
-  auto kern = k_bits_large<PACKED, DIRECT>;
+  auto kern = k_bits_large<PACKED, DICT>;
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBitSmem);
   note_launch();
   kern<<<blocks < n ? blocks : n, kLargeWarps * 32, kBitSmem, s>>>(
@@ -1036,8 +1049,8 @@ void launch_large(const DevGraph& g, const Oriented& o, const int32_t* list, int
 
 }  // namespace
 
-int64_t bits_slice_bytes(int64_t dmax, int64_t imax) {
-  return 16 * ((dmax + 15) / 16 * 16) + (2 * imax + 255) / 256 * 256;
+int64_t bits_slice_bytes(int64_t dmax, int64_t imax, int64_t nv) {
+  return 16 * ((dmax + 15) / 16 * 16) + (2 * imax + 255) / 256 * 256 + bits_val_bytes(nv);
 }
 
 cudaError_t launch_close_bits(int c, const DevGraph& g, const Oriented& o, int packed,
@@ -1064,8 +1077,9 @@ cudaError_t launch_close_bits(int c, const DevGraph& g, const Oriented& o, int p
     case 3: HG_SMALL(3); break;
     case 4: HG_SMALL(4); break;
     default:
-      if (g.nv <= kBitDirectVertices) HG_LARGE(true);
-      else HG_LARGE(false);
+      if (g.nv <= kBitDirectVertices) HG_LARGE(kDictDirect);
+      else if (g.nv <= kBitMapVertices) HG_LARGE(kDictMaps);
+      else HG_LARGE(kDictHash);
   }
 #undef HG_SMALL
 #undef HG_LARGE

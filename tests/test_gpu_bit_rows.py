@@ -27,11 +27,12 @@ def test_dense_small_teams(hglib, ne):
     check_against_oracle(hglib, 24, e_ptr, e_idx)
 
 
-@pytest.mark.parametrize("shift", [0, 40_000])
+@pytest.mark.parametrize("shift", [0, 40_000, 262_084, 300_000])
 def test_large_teams_direct_and_hash_dictionary(hglib, shift):
     # out-degrees up to 329 over hyperedges of 24-32 vertices: column lists beyond the
     # shared-memory teams, and more distinct row masks than the mask table holds; ids beyond
-    # the direct map's range send the same teams through the hash dictionary
+    # the direct map's range send the same teams through the maps with columns in scratch (up to
+    # 262,144 vertices) and the hash dictionary
     edges = random_edges(60, 330, 24, 32, 3)
     e_ptr, e_idx = csr_of([[v + shift for v in e] for e in edges])
     counts, st = check_against_oracle(hglib, 60 + shift, e_ptr, e_idx)
