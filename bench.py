@@ -205,10 +205,12 @@ def profiled_traffic(kernel, workload_name, units=None):
     return float(e["dram_bytes_per_launch"])
 
 
-# closure kernel groups: warp teams walking the out-lists, bit-row teams, global-table teams
-CLOSE_GROUPS = ("close_warp256", "close_warp512", "close_warp1024", "close_bits64", "close_bits128",
+# closure kernel groups: warp and block teams walking the out-lists, bit-row teams, global-table
+# teams
+CLOSE_GROUPS = ("close_warp256", "close_warp512", "close_warp1024", "close_block2048",
+                "close_block4096", "close_block8192", "close_bits64", "close_bits128",
                 "close_bits256", "close_bits512", "close_bits1024", "close_bits_large",
-                "close_wide", "close_cluster", "close_over")
+                "close_wide", "close_cluster")
 ISSUE_LANE_OPS_PER_CYCLE_PER_SM = 4 * 32   # 4 schedulers, one 32-lane instruction per cycle
 
 

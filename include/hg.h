@@ -88,9 +88,10 @@ typedef struct hg_tuning {
   int32_t dense_max_count; /* cap on the size of the dense set (0 = 1% of |E|) */
   int32_t close_mode;      /* step two team shape: 0 = by out-degree and |e_u| (warp
                               teams where they fit), 1 = global-table teams for every
-                              hyperedge, 2 = warp and bit-row teams build their
-                              tables, then hand every hyperedge over to the global-table
-                              teams (the path a team whose tables overflow takes);
+                              hyperedge, 2 = warp, block and bit-row teams build
+                              their tables, then hand every hyperedge over to the
+                              global-table teams (the path a team whose cuckoo stash
+                              overflows takes);
                               counts do not depend on it */
   int32_t orient_exact;    /* 1 = oriented rows in an exact layout (W entries, one extra
                               counting pass); 0 = room for deg(i) per row (2W entries)
@@ -100,7 +101,7 @@ typedef struct hg_tuning {
                                holds: 512 in the packed layout, 256 otherwise; 32..512,
                                capped at that largest) */
   int32_t warp_team_max;   /* step two: largest out-degree closed by a one-warp team; larger
-                              ones take bit-row teams (0 = 256; 64, 128 or 256) */
+                              ones take bit-row or block teams (0 = 256; 64, 128 or 256) */
   int32_t reserved[2];
 } hg_tuning;
 

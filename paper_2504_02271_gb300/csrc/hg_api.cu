@@ -1097,7 +1097,11 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
   g->counted = g->have_cstats = false;
   const int64_t ne = g->ne;
   Small h;
-  int32_t* lists = alloc_t<int32_t>(g, g->count_blocks, kLists * ne);
+  // Arrays of |E| owners, two lists in each where no owner can be in both: bit-row classes from
+  // both ends, a warp team's list and a block team's (bit-row teams append to these, but only
+  // owners of their label), the two kinds of global-table teams, the handed-over owners.
+  constexpr int kArrays = kBitClasses / 2 + 5;
+  int32_t* lists = alloc_t<int32_t>(g, g->count_blocks, kArrays * ne);
   if (!lists) return HG_ERR_OOM;
   uint8_t* sel = nullptr;
   if (h_sel) {
@@ -1120,8 +1124,15 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
     hist = g->mhist;
   }
   CloseLists cl;
-  for (int k = 0; k < kLists; ++k) cl.lists[k] = lists + k * ne;
-  cl.count = g->small->list_count;
+  auto two_lists = [&](int array, int up, int down) {
+    int32_t* base = lists + (int64_t)array * ne;
+    cl.list[up] = OwnerList{base, 1, g->small->list_count + up};
+    if (down >= 0) cl.list[down] = OwnerList{base + ne - 1, -1, g->small->list_count + down};
+  };
+  for (int k = 0; k < 3; ++k) two_lists(k, k, 3 + k);
+  two_lists(3, kListWide, kListCluster);
+  two_lists(4, kListOver, -1);
+  for (int k = 0; k < kBitClasses; k += 2) two_lists(5 + k / 2, kListBits + k, kListBits + k + 1);
   cl.labels = g->small->label_count;
   cl.maxima = g->small->close_max;
   DevGraph d = dev_graph(g);
@@ -1139,11 +1150,7 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
   int32_t n[kLists];
   for (int k = 0; k < kLists; ++k) n[k] = h.list_count[k];
   // scratch of the global-table teams: out-degrees and |e_u| up to the two maxima
-  struct Wide {
-    int64_t cap = 16, words = 1, dmax = 1;
-    void* scratch = nullptr;
-  };
-  auto wide_scratch = [&](unsigned long long dmax, unsigned long long smax, Wide* w) {
+  auto wide_scratch = [&](unsigned long long dmax, unsigned long long smax, WideSpace* w) {
     w->dmax = std::max<int64_t>((int64_t)dmax, 1);
     w->words = std::max<int64_t>(((int64_t)smax + 31) / 32, 1);
     while (w->cap < 2 * w->dmax) w->cap *= 2;
@@ -1151,9 +1158,7 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
                            close_wide_scratch_bytes(w->cap, w->words, w->dmax, g->nsm));
     return w->scratch != nullptr;
   };
-  Wide wide;
-  if (n[kListWide] + n[kListCluster] > 0 && !wide_scratch(h.close_max[0], h.close_max[1], &wide))
-    return HG_ERR_OOM;
+  WideSpace wide, over;
   const int64_t slice_dmax = ((int64_t)h.close_max[5] + 15) / 16 * 16;
   const int64_t slice = bits_slice_bytes(slice_dmax, (int64_t)h.close_max[4], g->nv);
   const int slice_blocks = std::min(n[kListBits + kBitClasses - 1], g->nsm);
@@ -1162,38 +1167,48 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
     slices = dev_alloc(g, g->count_blocks, (size_t)(slice * slice_blocks));
     if (!slices) return HG_ERR_OOM;
   }
-  static const char* names[kLists] = {"close_warp256",  "close_warp512",    "close_warp1024",
-                                      "close_bits64",   "close_bits128",    "close_bits256",
-                                      "close_bits512",  "close_bits1024",   "close_bits_large",
-                                      "close_wide",     "close_cluster",    "close_over"};
-  int32_t* overflow = cl.lists[kListOver];
-  int32_t* n_overflow = cl.count + kListOver;
-  for (int k = kListCluster; k >= 0; --k) {
+  static const char* names[kLists] = {
+      "close_warp256",  "close_warp512",   "close_warp1024",  "close_block2048", "close_block4096",
+      "close_block8192", "close_wide",     "close_cluster",   "close_bits64",    "close_bits128",
+      "close_bits256",  "close_bits512",   "close_bits1024",  "close_bits_large", "close_wide"};
+  const CloseRun run{d, g->ori, g->packed, hist, cl.list[kListOver], handover, s, g->nsm};
+  ReturnLists ret;
+  for (int k = 0; k < kCloseBuckets; ++k) ret.back[k] = cl.list[k];
+  int64_t n_bits = 0;
+  for (int k = kListOver - 1; k >= kListBits; --k) {
     if (n[k] <= 0) continue;
+    n_bits += n[k];
     t_begin(g, names[k]);
-    if (k >= kListBits && k < kListWide)
-      HG_CUDA(launch_close_bits(k - kListBits, d, g->ori, g->packed, cl.lists[k], n[k],
-                                cl.count + k, slices, slice, slice_dmax, slice_blocks, hist,
-                                &g->small->work[0][0], rule, g->small->counters + k, overflow,
-                                n_overflow, handover, s, g->nsm));
-    else
-      HG_CUDA(launch_close(k, d, g->ori, g->packed, cl.lists[k], n[k], cl.count + k, wide.cap,
-                           wide.words, wide.dmax, wide.scratch, hist,
-                           g->small->work[k == kListCluster ? kClusterBucket
-                                                            : (k == kListWide ? kWideBucket : k)],
-                           g->small->counters + k, overflow, n_overflow, handover, s, g->nsm));
+    HG_CUDA(launch_close_bits(k - kListBits, run, cl.list[k], n[k], ret, slices, slice, slice_dmax,
+                              slice_blocks, &g->small->work[0][0], rule, g->small->counters + k));
     t_end(g);
   }
+  // A walking team's list and what the bit-row teams gave back to it (`most`: an upper bound).
+  auto walk = [&](int k, int64_t most) {
+    if (k >= kListWide && k <= kListCluster && !wide.scratch &&
+        !wide_scratch(h.close_max[0], h.close_max[1], &wide))
+      return HG_ERR_OOM;
+    t_begin(g, names[k]);
+    HG_CUDA(launch_close(k, run, cl.list[k], (int32_t)std::min<int64_t>(most, ne),
+                         k == kListOver ? over : wide,
+                         g->small->work[k == kListOver ? kWideBucket : k], g->small->counters + k));
+    t_end(g);
+    return HG_OK;
+  };
+  for (int k = kListCluster; k >= 0; --k)
+    if (n[k] > 0) HG_TRY(walk(k, n[k] + n_bits));
   HG_TRY(sync_small(g, &h));
+  bool more = false;   // lists that were empty until a bit-row team gave an owner back
+  for (int k = kListCluster; k >= 0; --k)
+    if (n[k] <= 0 && h.list_count[k] > 0) {
+      HG_TRY(walk(k, h.list_count[k]));
+      more = true;
+    }
+  if (more) HG_TRY(sync_small(g, &h));
   const int32_t n_over = h.list_count[kListOver];
   if (n_over > 0) {
-    Wide over;
     if (!wide_scratch(h.close_max[2], h.close_max[3], &over)) return HG_ERR_OOM;
-    t_begin(g, "close_wide");
-    HG_CUDA(launch_close(kListOver, d, g->ori, g->packed, overflow, n_over, n_overflow, over.cap,
-                         over.words, over.dmax, over.scratch, hist, g->small->work[kWideBucket],
-                         g->small->counters + kListOver, overflow, n_overflow, 0, s, g->nsm));
-    t_end(g);
+    HG_TRY(walk(kListOver, n_over));
     HG_TRY(sync_small(g, &h));
   }
   t_collect(g);

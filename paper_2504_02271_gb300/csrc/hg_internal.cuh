@@ -264,25 +264,43 @@ struct TeamRule {
   }
 };
 
-// Lists: warp teams that walk the out-lists (labels 0-2), the bit-row classes, global-table
-// blocks, global-table clusters, and the owners no other list takes or that a team handed
-// over.
-constexpr int kListBits = 3;
+// Lists of owners: the walking teams by label (warp teams 0-2, block teams with shared tables
+// 3-5, global-table blocks and clusters), the bit-row classes, and the owners that a walking
+// team handed over to the global-table blocks.
+constexpr int kListWide = kWideBucket;
+constexpr int kListCluster = kClusterBucket;
+constexpr int kListBits = kCloseBuckets;
 constexpr int kBitClasses = 6;
-constexpr int kListWide = kListBits + kBitClasses;
-constexpr int kListCluster = kListWide + 1;
-constexpr int kListOver = kListCluster + 1;
+constexpr int kListOver = kListBits + kBitClasses;
 constexpr int kLists = kListOver + 1;
+
+// A list of owners on the device: entry k at at[k * step], its length at *n.  Two lists share
+// an array of |E| entries where no owner can be in both, one from each end.
+struct OwnerList {
+  int32_t* at;
+  int32_t step;
+  int32_t* n;
+#ifdef __CUDACC__
+  __device__ __forceinline__ int32_t get(int32_t k) const { return at[(int64_t)k * step]; }
+  __device__ __forceinline__ void put(int32_t u) const {
+    at[(int64_t)atomicAdd(n, 1) * step] = u;
+  }
+#endif
+};
 constexpr int kWalkRatio0 = 8, kWalkRatio3 = 40, kWalkRatio4 = 80;   // see list_of in k_close.cu
 constexpr int kBitMaxOut = 8192;             // bit rows: out-degree, column-list entries
 constexpr int kBitMaxEntries = 1 << 22;
 // Direct vertex map up to kBitDirectVertices; its bit maps alone in shared memory up to
-// kBitMapVertices (at most 64 KB, less than the hash), its columns in global scratch.  The hash
-// holds 16,384 vertices and an owner with more goes to the global-table blocks: closure of a
-// tag shape of 200,000 hyperedges over 40,000 vertices 1.56 against 0.35 s, of 300,000 over
-// 100,000 3.79 against 0.52 (the block teams before: 1.08, 1.57).
+// kBitMapVertices (at most 64 KB, less than the hash), its columns in global scratch.  Beyond,
+// a hash of 16,384 vertices: closure of a tag shape of 200,000 hyperedges over 40,000 vertices
+// 1.56 with the hash and 0.35 s with the maps, of 300,000 over 100,000 3.79 and 0.52 (block
+// teams: 1.08, 1.57).  An owner that fills the hash goes to the block teams after its vertices
+// were read, so the hash is tried up to kBitHashEntries of osum + |e_u| (closure of 60,000 and
+// 300,000 tag-shaped hyperedges over 300,000 vertices, ms: never 195, 1,389; 16,384 190, 1,356;
+// 32,768 155, 1,170; 65,536 126, 1,248; 131,072 130, 1,441).
 constexpr int kBitDirectVertices = 32768;
 constexpr int kBitMapVertices = 262144;
+constexpr int kBitHashEntries = 65536;
 
 constexpr int kBitSmem = 232448 - 2048;      // dynamic shared memory a block may take
 constexpr int kBitPlanes = 16;               // digits of a shared count (<= 65,535)
@@ -322,36 +340,48 @@ __host__ __device__ inline int bit_class_of(int64_t du, int64_t szu, int64_t osu
 
 // k_close.cu
 struct CloseLists {
-  int32_t* lists[kLists];
-  int32_t* count;         // [kLists]
+  OwnerList list[kLists];
   int32_t* labels;        // [kCloseBuckets] owners per label
-  unsigned long long* maxima;   // largest [0] out-degree, [1] |e_u| of the wide and cluster
-                                // lists, [2], [3] of all, [4] osum, [5] out-degree of the
+  unsigned long long* maxima;   // largest [0] out-degree, [1] |e_u| of the labels 6 and 7,
+                                // [2], [3] of the others, [4] osum, [5] out-degree of the
                                 // last bit class
 };
 // sel: NULL, or one byte per hyperedge; then only the hyperedges u with sel[u] != 0
 // get a team (the hyper-triangles they own).
 void launch_bucket_close(const DevGraph& g, const Oriented& o, CloseLists b, const TeamRule& rule,
                          const uint8_t* sel, cudaStream_t s);
-// list: 0, 1, 2 (warp teams by label), kListWide, kListCluster or kListOver; n: its length
-// (host copy); n_p: the same on the device; counter: zeroed fetch counter; work[0] += probes,
-// work[1] += E_y entries, work[2] += out-entries (hg_close_stats); the warp teams append
-// owners their tables cannot hold (every one when handover is set) to
-// overflow[*n_overflow++]
-cudaError_t launch_close(int list_id, const DevGraph& g, const Oriented& o, int packed,
-                  const int32_t* list, int32_t n, const int32_t* n_p, int64_t wide_cap,
-                  int64_t wide_words, int64_t wide_dmax, void* scratch, unsigned long long* hist,
-                  unsigned long long* work, int32_t* counter, int32_t* overflow,
-                  int32_t* n_overflow, int handover, cudaStream_t s, int nsm);
+// What every kernel of a count shares.
+struct CloseRun {
+  DevGraph g;
+  Oriented o;
+  int packed;
+  unsigned long long* hist;
+  OwnerList over;   // owners that the walking teams' tables cannot hold (every one of the warp,
+  int handover;     // block and bit-row teams when handover is set)
+  cudaStream_t s;
+  int nsm;
+};
+// Scratch of the global-table teams.
+struct WideSpace {
+  int64_t cap = 16, words = 1, dmax = 1;
+  void* scratch = nullptr;
+};
+// list_id: a walking team's list or kListOver; n: its length, or an upper bound (sizes the
+// grid; the kernel reads the length on the device); counter: zeroed fetch counter; work[0] +=
+// probes, work[1] += E_y entries, work[2] += out-entries (hg_close_stats)
+cudaError_t launch_close(int list_id, const CloseRun& r, const OwnerList& list, int32_t n,
+                         const WideSpace& w, unsigned long long* work, int32_t* counter);
 // k_bits.cu: the owners of bit-row class c.  work: [kCloseBuckets][3] as above, by label.
-// The last class keeps `slice` bytes of scratch per block, at most blocks_max blocks.
+// back[label]: the walking team's list that an owner whose tables overflow goes to.  The last
+// class keeps `slice` bytes of scratch per block, at most blocks_max blocks.
+struct ReturnLists {
+  OwnerList back[kCloseBuckets];
+};
 int64_t bits_slice_bytes(int64_t dmax, int64_t imax, int64_t nv);
-cudaError_t launch_close_bits(int c, const DevGraph& g, const Oriented& o, int packed,
-                       const int32_t* list, int32_t n, const int32_t* n_p, void* scratch,
-                       int64_t slice, int64_t dmax, int blocks_max, unsigned long long* hist,
-                       unsigned long long* work, const TeamRule& rule, int32_t* counter,
-                       int32_t* overflow, int32_t* n_overflow, int handover, cudaStream_t s,
-                       int nsm);
+cudaError_t launch_close_bits(int c, const CloseRun& r, const OwnerList& list, int32_t n,
+                              const ReturnLists& ret, void* scratch, int64_t slice, int64_t dmax,
+                              int blocks_max, unsigned long long* work, const TeamRule& rule,
+                              int32_t* counter);
 size_t close_wide_scratch_bytes(int64_t cap, int64_t words, int64_t dmax, int nsm);
 
 }  // namespace hg

@@ -70,7 +70,7 @@ struct Dict {
   uint16_t* val;
   int log2;
   int words;
-  // *full is set when a key finds no slot within kMaxProbes (the team is then handed over)
+  // *full is set when a key finds no slot within kMaxProbes (the owner is then given back)
   __device__ __forceinline__ uint32_t touch(uint32_t y, int* ncol, int* full) const {
     if (DIRECT) {
       const uint32_t b = 1u << (y & 31u);
@@ -412,18 +412,28 @@ struct SmallLayout {
 struct NextOwner {
   int32_t r, u;
   __device__ __forceinline__ void fetch(int32_t* counter) { r = atomicAdd(counter, 1); }
-  __device__ __forceinline__ void find(const int32_t* list, int32_t n) {
-    u = r < n ? __ldg(list + r) : -1;
+  __device__ __forceinline__ void find(const OwnerList& list, int32_t n) {
+    u = r < n ? list.get(r) : -1;
   }
 };
 
+// An owner that a team cannot hold goes back to the walking team of its label (to the
+// global-table blocks when every owner is to be handed over).
+__device__ __forceinline__ void give_back(const ReturnLists& ret, const OwnerList& handed,
+                                          int handover, int label, int32_t u) {
+  const bool all = handover && label < kWideBucket;
+#pragma unroll
+  for (int k = 0; k < kCloseBuckets; ++k)   // (the lists are kernel parameters: no indexing)
+    if (!all && k == label) ret.back[k].put(u);
+  if (all) handed.put(u);
+}
+
 template <int NW, int MINB, bool PACKED, typename ROW>
 __global__ void __launch_bounds__(NW * 32, MINB)
-    k_bits_small(DevGraph g, Oriented o, SmallLayout ly, const int32_t* __restrict__ list,
-                 const int32_t* __restrict__ n_p, unsigned long long* __restrict__ hist_out,
-                 unsigned long long* __restrict__ work, TeamRule rule,
-                 int32_t* __restrict__ counter, int32_t* __restrict__ overflow,
-                 int32_t* __restrict__ n_overflow, int handover) {
+    k_bits_small(DevGraph g, Oriented o, SmallLayout ly, OwnerList list,
+                 unsigned long long* __restrict__ hist_out, unsigned long long* __restrict__ work,
+                 TeamRule rule, int32_t* __restrict__ counter, ReturnLists ret, OwnerList handed,
+                 int handover) {
   constexpr int NT = NW * 32, G = 4;
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ TeamBlock tb;
@@ -450,7 +460,7 @@ __global__ void __launch_bounds__(NW * 32, MINB)
   uint32_t* S = reinterpret_cast<uint32_t*>(dyn + ly.off_s);
   for (int k = tid; k < kBins; k += NT) tb.hist[k] = 0;
   for (int k = tid; k < kCloseBuckets * 3; k += NT) (&tb.work[0][0])[k] = 0;
-  const int32_t n = *n_p;
+  const int32_t n = *list.n;
   uint32_t cls[kClasses];
 #pragma unroll
   for (int q = 0; q < kClasses; ++q) cls[q] = 0;
@@ -606,8 +616,8 @@ __global__ void __launch_bounds__(NW * 32, MINB)
       while (cw > 1 && scol * cw > ly.swords) cw >>= 1;
     }
     const bool over = handover || tb.full != 0 || scol * cw > ly.swords;
-    if (over) {   // the same on every thread: the global-table teams take u
-      if (tid == 0) overflow[atomicAdd(n_overflow, 1)] = u;
+    if (over) {   // the same on every thread: a walking team takes u
+      if (tid == 0) give_back(ret, handed, handover, rule.label(du, szu), u);
     } else {
       for (int k = tid; k < scol * cw; k += NT) S[k] = 0;
       team_sync<NW>();
@@ -734,12 +744,11 @@ enum { kDictHash, kDictDirect, kDictMaps };
 
 template <bool PACKED, int DICT>
 __global__ void __launch_bounds__(kLargeWarps * 32, 1)
-    k_bits_large(DevGraph g, Oriented o, int slots_log2, const int32_t* __restrict__ list,
-                 const int32_t* __restrict__ n_p, char* __restrict__ scratch, int64_t slice,
-                 int64_t dmax, unsigned long long* __restrict__ hist_out,
-                 unsigned long long* __restrict__ work, TeamRule rule,
-                 int32_t* __restrict__ counter, int32_t* __restrict__ overflow,
-                 int32_t* __restrict__ n_overflow, int handover) {
+    k_bits_large(DevGraph g, Oriented o, int slots_log2, OwnerList list,
+                 char* __restrict__ scratch, int64_t slice, int64_t dmax,
+                 unsigned long long* __restrict__ hist_out, unsigned long long* __restrict__ work,
+                 TeamRule rule, int32_t* __restrict__ counter, ReturnLists ret, OwnerList handed,
+                 int handover) {
   constexpr int NW = kLargeWarps, NT = NW * 32, G = 8;
   constexpr bool DIRECT = DICT != kDictHash;
   extern __shared__ __align__(16) unsigned char dyn[];
@@ -751,7 +760,7 @@ __global__ void __launch_bounds__(kLargeWarps * 32, 1)
                                                bits_val_bytes(g.nv));
   for (int k = tid; k < kBins; k += NT) tb.hist[k] = 0;
   for (int k = tid; k < kCloseBuckets * 3; k += NT) (&tb.work[0][0])[k] = 0;
-  const int32_t n = *n_p;
+  const int32_t n = *list.n;
   uint32_t cls[kClasses];
 #pragma unroll
   for (int q = 0; q < kClasses; ++q) cls[q] = 0;
@@ -865,7 +874,7 @@ __global__ void __launch_bounds__(kLargeWarps * 32, 1)
     if (!over) {
       // 2. shared vertices
       for_each_row<NW>(g, src, du, lane, w, [&](int, uint32_t, int32_t v) {
-        // (once it is full, every further vertex would take all its probes for nothing)
+        // (once a hash is full, every further vertex would take all its probes for nothing)
         if (v >= 0 && (DIRECT || !*(volatile int*)&tb.full))
           dict.touch((uint32_t)v, &tb.ncol, &tb.full);
       });
@@ -916,7 +925,7 @@ __global__ void __launch_bounds__(kLargeWarps * 32, 1)
       over = cw < 1;
     }
     if (over) {
-      if (tid == 0) overflow[atomicAdd(n_overflow, 1)] = u;
+      if (tid == 0) give_back(ret, handed, handover, rule.label(du, szu), u);
     } else {
       if (tid == 0) {
         const int label = rule.label(du, szu);
@@ -1013,10 +1022,8 @@ constexpr SmallLayout small_layout(int c) {
 }
 
 template <int C, bool PACKED>
-void launch_small(const DevGraph& g, const Oriented& o, const int32_t* list, int32_t n,
-                  const int32_t* n_p, unsigned long long* hist, unsigned long long* work,
-                  const TeamRule& rule, int32_t* counter, int32_t* overflow,
-                  int32_t* n_overflow, int handover, cudaStream_t s, int nsm) {
+void launch_small(const CloseRun& r, const OwnerList& list, int32_t n, const ReturnLists& ret,
+                  unsigned long long* work, const TeamRule& rule, int32_t* counter) {
   constexpr Shape sh = kShapes[C];
   using ROW = typename std::conditional<(sh.dcap <= 256), uint8_t, uint16_t>::type;
   auto kern = k_bits_small<sh.nw, sh.minb, PACKED, ROW>;
@@ -1027,24 +1034,22 @@ void launch_small(const DevGraph& g, const Oriented& o, const int32_t* list, int
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, sh.nw * 32, ly.bytes);
   if (per_sm < 1) per_sm = 1;
-  const int blocks = n < per_sm * nsm ? n : per_sm * nsm;
+  const int blocks = n < per_sm * r.nsm ? n : per_sm * r.nsm;
   note_launch();
-  kern<<<blocks, sh.nw * 32, ly.bytes, s>>>(g, o, ly, list, n_p, hist, work, rule, counter,
-                                            overflow, n_overflow, handover);
+  kern<<<blocks, sh.nw * 32, ly.bytes, r.s>>>(r.g, r.o, ly, list, r.hist, work, rule, counter, ret,
+                                              r.over, r.handover);
 }
 
 template <bool PACKED, int DICT>
-void launch_large(const DevGraph& g, const Oriented& o, const int32_t* list, int32_t n,
-                  const int32_t* n_p, void* scratch, int64_t slice, int64_t dmax, int blocks,
-                  unsigned long long* hist, unsigned long long* work, const TeamRule& rule,
-                  int32_t* counter, int32_t* overflow, int32_t* n_overflow, int handover,
-                  cudaStream_t s) {
+void launch_large(const CloseRun& r, const OwnerList& list, int32_t n, const ReturnLists& ret,
+                  void* scratch, int64_t slice, int64_t dmax, int blocks,
+                  unsigned long long* work, const TeamRule& rule, int32_t* counter) {
   auto kern = k_bits_large<PACKED, DICT>;
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBitSmem);
   note_launch();
-  kern<<<blocks < n ? blocks : n, kLargeWarps * 32, kBitSmem, s>>>(
-      g, o, kBitLargeSlots, list, n_p, (char*)scratch, slice, dmax, hist, work, rule, counter, overflow,
-      n_overflow, handover);
+  kern<<<blocks < n ? blocks : n, kLargeWarps * 32, kBitSmem, r.s>>>(
+      r.g, r.o, kBitLargeSlots, list, (char*)scratch, slice, dmax, r.hist, work, rule, counter, ret,
+      r.over, r.handover);
 }
 
 }  // namespace
@@ -1053,23 +1058,19 @@ int64_t bits_slice_bytes(int64_t dmax, int64_t imax, int64_t nv) {
   return 16 * ((dmax + 15) / 16 * 16) + (2 * imax + 255) / 256 * 256 + bits_val_bytes(nv);
 }
 
-cudaError_t launch_close_bits(int c, const DevGraph& g, const Oriented& o, int packed,
-                       const int32_t* list, int32_t n, const int32_t* n_p, void* scratch,
-                       int64_t slice, int64_t dmax, int blocks_max, unsigned long long* hist,
-                       unsigned long long* work, const TeamRule& rule, int32_t* counter,
-                       int32_t* overflow, int32_t* n_overflow, int handover, cudaStream_t s,
-                       int nsm) {
+cudaError_t launch_close_bits(int c, const CloseRun& r, const OwnerList& list, int32_t n,
+                              const ReturnLists& ret, void* scratch, int64_t slice, int64_t dmax,
+                              int blocks_max, unsigned long long* work, const TeamRule& rule,
+                              int32_t* counter) {
   if (n <= 0) return cudaSuccess;
-#define HG_SMALL(C)                                                                            \
-  (packed ? launch_small<C, true>(g, o, list, n, n_p, hist, work, rule, counter, overflow,     \
-                                  n_overflow, handover, s, nsm)                                \
-          : launch_small<C, false>(g, o, list, n, n_p, hist, work, rule, counter, overflow,    \
-                                   n_overflow, handover, s, nsm))
-#define HG_LARGE(D)                                                                            \
-  (packed ? launch_large<true, D>(g, o, list, n, n_p, scratch, slice, dmax, blocks_max, hist,  \
-                                  work, rule, counter, overflow, n_overflow, handover, s)      \
-          : launch_large<false, D>(g, o, list, n, n_p, scratch, slice, dmax, blocks_max, hist, \
-                                   work, rule, counter, overflow, n_overflow, handover, s))
+#define HG_SMALL(C)                                                                     \
+  (r.packed ? launch_small<C, true>(r, list, n, ret, work, rule, counter)               \
+            : launch_small<C, false>(r, list, n, ret, work, rule, counter))
+#define HG_LARGE(D)                                                                              \
+  (r.packed ? launch_large<true, D>(r, list, n, ret, scratch, slice, dmax, blocks_max, work, rule, \
+                                    counter)                                                     \
+            : launch_large<false, D>(r, list, n, ret, scratch, slice, dmax, blocks_max, work,    \
+                                     rule, counter))
   switch (c) {
     case 0: HG_SMALL(0); break;
     case 1: HG_SMALL(1); break;
@@ -1077,8 +1078,8 @@ cudaError_t launch_close_bits(int c, const DevGraph& g, const Oriented& o, int p
     case 3: HG_SMALL(3); break;
     case 4: HG_SMALL(4); break;
     default:
-      if (g.nv <= kBitDirectVertices) HG_LARGE(kDictDirect);
-      else if (g.nv <= kBitMapVertices) HG_LARGE(kDictMaps);
+      if (r.g.nv <= kBitDirectVertices) HG_LARGE(kDictDirect);
+      else if (r.g.nv <= kBitMapVertices) HG_LARGE(kDictMaps);
       else HG_LARGE(kDictHash);
   }
 #undef HG_SMALL

@@ -88,7 +88,7 @@ __device__ __forceinline__ uint32_t full_mask(int sz) { return sz >= 32 ? ~0u : 
 // classification runs with every lane active.
 
 // Entries of out(v) loaded per lane before their probes (loads in flight per warp):
-// warp_unroll(D_LOG2).  On the
+// warp_unroll(D_LOG2) in the warp teams, kBlockUnroll in the block teams.  On the
 // co-authorship workload the out-degree-128 teams were fastest with 6 (6.01 ms; 8: 6.13,
 // 10: 6.09), the out-degree-64 and -256 ones with 10 (0.875 and 1.184 ms; 8: 0.885 and
 // 1.198).  HG_CLOSE_WARP_UNROLL sets one value for all three.
@@ -97,6 +97,18 @@ __host__ __device__ constexpr int warp_unroll(int) { return HG_CLOSE_WARP_UNROLL
 #else
 __host__ __device__ constexpr int warp_unroll(int d_log2) { return d_log2 == 7 ? 6 : 10; }
 #endif
+// Warps of a block team (one block per SM: shared memory holds one team's tables).  On
+// a tag-shaped prefix of 500,000 hyperedges 16, 24 and 32 warps took 7.22, 5.73 and 5.16 s
+// per step with these teams alone.  The unpacked layout's hit queue is 4x wider, so it keeps
+// to 24 warps (its out-degree-4096 tables with 32 warps would leave under 2 KB of the 227 KB
+// that a block may use).
+#ifndef HG_BLOCK_WARPS
+#define HG_BLOCK_WARPS 32
+#endif
+constexpr int kBlockWarps = HG_BLOCK_WARPS;
+constexpr int kBlockWarpsUnpacked = HG_BLOCK_WARPS < 24 ? HG_BLOCK_WARPS : 24;
+constexpr int kBlockUnroll = 8;
+constexpr int kQueue = 32 * kBlockUnroll + 32;
 constexpr int kCuckooTries = 16;
 constexpr int kStash = 8;
 
@@ -162,6 +174,35 @@ __device__ __forceinline__ int warp_find(const TT& t, int32_t x, int nst) {
   }
   return m < 256 ? (int)m : -1;
 }
+
+// Start of out(x)'s entries in the oriented rows: a pointer per layout, so that a probe
+// addresses entry j of the current row with one 32-bit index.
+template <bool PACKED>
+struct RowPtr {
+  const uint32_t* p;   // packed entries
+  const int32_t* n;    // unpacked: neighbour ids
+  const int32_t* w;    // unpacked: omega
+  __device__ __forceinline__ void at(const Oriented& o, int64_t off) {
+    if (PACKED) {
+      p = o.packed + off;
+    } else {
+      n = o.nbr + off;
+      w = o.omega + off;
+    }
+  }
+  __device__ __forceinline__ void load(int32_t j, int32_t& nbr, int32_t& om) const {
+    if (PACKED) {
+      const uint32_t x = __ldg(p + j);
+      nbr = (int32_t)(x >> 8);
+      om = (int32_t)(x & 0xffu);
+    } else {
+      nbr = __ldg(n + j);
+      om = __ldg(w + j);
+    }
+  }
+  // packed layout only: the entry as stored, (nbr << 8) | omega
+  __device__ __forceinline__ uint32_t raw(int32_t j) const { return __ldg(p + j); }
+};
 
 __device__ __forceinline__ uint32_t filt_bit(uint32_t key, int bits_log2) {
   return (key * 0x85EBCA6Bu) >> (32 - bits_log2);
@@ -304,10 +345,9 @@ __host__ __device__ constexpr int warp_threads_per_sm(int d_log2) {
 
 template <int D_LOG2, int WARPS, bool PACKED, bool OFF32>
 __global__ void __launch_bounds__(WARPS * 32, warp_threads_per_sm(D_LOG2) / (WARPS * 32))
-    k_close_warp(DevGraph g, Oriented o, const int32_t* __restrict__ list,
-                 const int32_t* __restrict__ n_p, unsigned long long* __restrict__ hist_out,
-                 unsigned long long* __restrict__ work, int32_t* __restrict__ counter,
-                 int32_t* __restrict__ overflow, int32_t* __restrict__ n_overflow, int handover) {
+    k_close_warp(DevGraph g, Oriented o, OwnerList list,
+                 unsigned long long* __restrict__ hist_out, unsigned long long* __restrict__ work,
+                 int32_t* __restrict__ counter, OwnerList over, int handover) {
   using TT = WarpTables<D_LOG2, PACKED, OFF32>;
   using Item = typename TT::Item;
   constexpr int T = TT::T, T_LOG2 = TT::T_LOG2;
@@ -318,7 +358,7 @@ __global__ void __launch_bounds__(WARPS * 32, warp_threads_per_sm(D_LOG2) / (WAR
   TT& t = tabs[w];
   for (int k = lane; k < kBins; k += 32) hist[w][k] = 0;
   __syncthreads();
-  const int32_t n = *n_p;
+  const int32_t n = *list.n;
   RunHist rh;
   unsigned long long probes = 0, gathers = 0, outs = 0, since_flush = 0;
   int32_t cur = 0;   // member whose bins the shared histogram holds
@@ -328,7 +368,7 @@ __global__ void __launch_bounds__(WARPS * 32, warp_threads_per_sm(D_LOG2) / (WAR
     if (lane == 0) r = atomicAdd(counter, 1);
     r = __shfl_sync(kFull, r, 0);
     if (r >= n) break;
-    const int32_t u = list[r];
+    const int32_t u = list.get(r);
     const int32_t m = member_of(g, u);
     if (m != cur || since_flush > (1ull << 30)) {   // 32-bit bins stay far from overflow
       warp_flush(rh, hist[w], hist_out + (size_t)cur * kBins, lane);
@@ -382,7 +422,7 @@ __global__ void __launch_bounds__(WARPS * 32, warp_threads_per_sm(D_LOG2) / (WAR
     __syncwarp();
     const int nst = *((volatile int32_t*)&t.nstash);
     if (nst > kStash || handover) {   // warp-uniform: the global-table teams take u
-      if (lane == 0) overflow[atomicAdd(n_overflow, 1)] = u;
+      if (lane == 0) over.put(u);
       __syncwarp();
       continue;
     }
@@ -457,19 +497,345 @@ __global__ void __launch_bounds__(WARPS * 32, warp_threads_per_sm(D_LOG2) / (WAR
   }
 }
 
-// ------------------------------------------------------------------ block per u (wide)
-// Any |e_u| (masks of `words` 32-bit words) and any out-degree; tables in global scratch.
+// ------------------------------------------------------------------ block per u (shared tables)
+//
+// One block owns one hyperedge u with |e_u| <= 32 and out-degree <= D.  out(u)
+// is a two-table cuckoo set with 2D slots per table.  A slot stores a key by
+// quotient: with the odd multiplier A of its table, p = x A mod 2^32 is a
+// bijection of x, the top T_LOG2 bits of p are the slot and the remaining
+// 31 - D_LOG2 bits are stored beside the index k of x in out(u), so 31 bits
+// identify (x, k) exactly and the top bit marks an empty slot.  An evicted key
+// is recovered from its slot and remainder with the inverse of A.  Keys not
+// placed within kCuckooTries evictions go to a stash; a team whose stash
+// overflows is handed to the global-table teams.  Per-k arrays hold the Omega_ux
+// mask, |e_x|, and the place and prefix-summed length of out(x).  The flat range
+// of all out(v) entries is cut into WARPS slices of equal length; each warp walks
+// its slice like the warp kernel (32 consecutive entries per load, lookup, queue,
+// 32-wide classification).
+//
+// These teams take the owners of out-degree above a warp team's that bit rows cannot hold,
+// by rule (list_of) or because a bit-row team's tables overflow.  The global-table blocks
+// need 2-3 times as long for them.  Closure, these teams alone / global-table blocks in their
+// place / these (ms): 60,000 tag-shaped hyperedges over 300,000 vertices 199 / 223 / 126,
+// 300,000 of them 1,406 / 3,481 / 1,250; 8,000 hyperedges of 20-32 out of 100 vertices beside
+// 50,000 unused ones (out-degrees up to 7,972) 548 / 522 / 486.
 
-// Slots of the global tables store a key by quotient: with the odd multiplier A of its
-// table, p = x A mod 2^32 is a bijection of x, the top bits of p are the slot and the
-// others are stored beside the index k of x in out(u).  An evicted key is recovered from
-// its slot and remainder with the inverse of A.
 constexpr uint32_t kCuckooA1 = 0x9E3779B1u, kCuckooA1Inv = 0x0E8B2F51u;
 constexpr uint32_t kCuckooA2 = 0x85EBCA6Bu, kCuckooA2Inv = 0xA5CB9243u;
 static_assert(kCuckooA1 * kCuckooA1Inv == 1u && kCuckooA2 * kCuckooA2Inv == 1u,
               "multiplicative inverses mod 2^32");
 
-// Per block: out(u) as a two-table cuckoo set coded by quotient
+// DMAX below 2^D_LOG2 (the 6,144 shape): indices keep D_LOG2 bits, each table has
+// 2^D_LOG2 slots (at most 3/8 of both tables in use), and a slot's remainder and index
+// fill all 32 bits; the empty word (all ones) still matches no key, because its index
+// field (all ones) is at least DMAX.
+template <int D_LOG2, int WARPS, bool PACKED, int DMAX = (1 << D_LOG2)>
+struct alignas(16) BlockTables {
+  static constexpr int D = DMAX;
+  static constexpr int T_LOG2 = DMAX == (1 << D_LOG2) ? D_LOG2 + 1 : D_LOG2;
+  static constexpr int T = 1 << T_LOG2;
+  static_assert(DMAX == (1 << D_LOG2) || (DMAX < (1 << D_LOG2) && 4 * DMAX <= 3 * (1 << D_LOG2)),
+                "a smaller DMAX keeps the tables at most 3/8 full");
+  uint32_t c1[T];
+  uint32_t c2[T];
+  int32_t skey[kStash];
+  int32_t sidx[kStash];
+  int64_t kbeg[D];
+  int32_t kpre[D + 1];       // exclusive prefix of the out-degrees of out(u)
+  uint32_t kmask[D];
+  uint16_t ksz[D];           // |e_x|, then |e_x| - omega_ux once masks are built
+  uint32_t queue[WARPS][kQueue];   // hits: (k_v << 16) | k_w ; omega in qom
+  uint8_t qom8[PACKED ? WARPS : 1][PACKED ? kQueue : 1];
+  int32_t qom[PACKED ? 1 : WARPS][PACKED ? 1 : kQueue];
+  int64_t ylen[32], yincl[32], ybeg[32];
+  int32_t nstash;
+};
+
+// Index k in out(u) of hyperedge x, or -1 (x = -1 matches nothing: keys are < 2^31).
+template <int D_LOG2, int WARPS, bool PACKED, int DMAX, bool STASH = true>
+__device__ __forceinline__ int block_find(const BlockTables<D_LOG2, WARPS, PACKED, DMAX>& t,
+                                          int32_t x, int nst) {
+  constexpr int SH = 32 - BlockTables<D_LOG2, WARPS, PACKED, DMAX>::T_LOG2;   // remainder bits
+  constexpr uint32_t RM = (1u << SH) - 1u;
+  const uint32_t p1 = (uint32_t)x * kCuckooA1, p2 = (uint32_t)x * kCuckooA2;
+  // an item (remainder << D_LOG2) | k xor-ed with the key's remainder so shifted is k
+  // (< DMAX) when the remainders agree, and at least 2^D_LOG2 otherwise; an empty slot
+  // gives at least DMAX (the top bit, or an index field of all ones); a key sits in at
+  // most one table
+  const uint32_t a = t.c1[p1 >> SH] ^ ((p1 & RM) << D_LOG2);
+  const uint32_t b = t.c2[p2 >> SH] ^ ((p2 & RM) << D_LOG2);
+  const uint32_t m = a < b ? a : b;
+  int k = m < (uint32_t)DMAX ? (int)m : -1;
+  if (STASH)
+    for (int i = 0; i < nst; ++i) k = t.skey[i] == x ? t.sidx[i] : k;
+  return k;
+}
+
+// Step 3 of a block team, for warp w: the slice [f_lo, f_hi) of the flat range of all
+// out(v), v in out(u), walked like the warp teams' (kBlockUnroll loads in flight, a
+// cursor per lane, queued 32-wide classification); the slice start is found by a
+// binary search over the prefix sums kpre of the out-degrees.
+template <int D_LOG2, int WARPS, bool PACKED, int DMAX, bool STASH>
+__device__ __forceinline__ void block_walk(BlockTables<D_LOG2, WARPS, PACKED, DMAX>& t,
+                                           const Oriented& o, int32_t u, int32_t du,
+                                           int32_t f_lo, int32_t f_hi, int nst, uint32_t fu,
+                                           uint32_t* hist, RunHist& rh, int lane, int w) {
+  int qn = 0;
+  uint32_t* queue = t.queue[w];
+  // cursor of this lane: first entry f_lo + lane -> (ck, cj); past the slice: ck = du
+  int ck = du, cj = 0, ccnt = INT32_MAX;
+  RowPtr<PACKED> rp;
+  rp.at(o, 0);
+  {
+    const int32_t f0 = f_lo + lane;
+    int lo = 0, hi = du;   // last k with kpre[k] <= f0
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (t.kpre[mid] <= f0) lo = mid; else hi = mid - 1;
+    }
+    if (f0 < f_hi && lo < du) {
+      ck = lo;
+      cj = f0 - t.kpre[ck];
+      ccnt = t.kpre[ck + 1] - t.kpre[ck];
+      rp.at(o, t.kbeg[ck]);
+    }
+  }
+  for (int32_t base = f_lo; base < f_hi; base += 32 * kBlockUnroll) {
+    int32_t ent_w[kBlockUnroll], ent_om[PACKED ? 1 : kBlockUnroll], ent_k[kBlockUnroll];
+#pragma unroll
+    for (int q = 0; q < kBlockUnroll; ++q) {
+      ent_k[q] = ck;
+      const bool in = ck < du && base + q * 32 + lane < f_hi;
+      if (PACKED) {
+        ent_w[q] = (int32_t)((uint32_t)u << 8);   // no entry: u, never in out(u)
+        if (in) ent_w[q] = (int32_t)rp.raw(cj);
+      } else {
+        ent_w[q] = u;
+        ent_om[q] = 0;
+        if (in) rp.load(cj, ent_w[q], ent_om[q]);
+      }
+      cj += 32;
+      if (cj >= ccnt) {
+        do {
+          cj -= ccnt;
+          ++ck;
+          ccnt = ck < du ? t.kpre[ck + 1] - t.kpre[ck] : INT32_MAX;
+        } while (cj >= ccnt);
+        if (ck < du) rp.at(o, t.kbeg[ck]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kBlockUnroll; ++q) {
+      const int32_t x = PACKED ? (int32_t)((uint32_t)ent_w[q] >> 8) : ent_w[q];
+      const int kw = block_find<D_LOG2, WARPS, PACKED, DMAX, STASH>(t, x, nst);
+      const bool hit = kw >= 0;
+      const unsigned bal = __ballot_sync(kFull, hit);
+      if (hit) {
+        const int at = qn + __popc(bal & ((1u << lane) - 1u));
+        queue[at] = ((uint32_t)ent_k[q] << 16) | (uint32_t)kw;
+        if (PACKED) t.qom8[w][at] = (uint8_t)((uint32_t)ent_w[q] & 0xffu);
+        else t.qom[w][at] = ent_om[PACKED ? 0 : q];
+      }
+      qn += __popc(bal);
+    }
+    __syncwarp();
+    while (qn >= 32) {
+      qn -= 32;
+      const int at = qn + lane;
+      const uint32_t e = queue[at];
+      const uint32_t kv = e >> 16, kw = e & 0xffffu;
+      const int om = PACKED ? (int)t.qom8[w][at] : t.qom[w][at];
+      rh.add(region_bits(fu, t.kmask[kv], t.kmask[kw], t.ksz[kv], t.ksz[kw], om), hist);
+      __syncwarp();
+    }
+  }
+  if (lane < qn) {
+    const uint32_t e = queue[lane];
+    const uint32_t kv = e >> 16, kw = e & 0xffffu;
+    const int om = PACKED ? (int)t.qom8[w][lane] : t.qom[w][lane];
+    rh.add(region_bits(fu, t.kmask[kv], t.kmask[kw], t.ksz[kv], t.ksz[kw], om), hist);
+  }
+  __syncwarp();
+}
+
+template <int D_LOG2, int WARPS, bool PACKED, int DMAX>
+__global__ void __launch_bounds__(WARPS * 32, 1)
+    k_close_block(DevGraph g, Oriented o, OwnerList list,
+                  unsigned long long* __restrict__ hist_out, unsigned long long* __restrict__ work,
+                  int32_t* __restrict__ counter, OwnerList over, int handover) {
+  using TT = BlockTables<D_LOG2, WARPS, PACKED, DMAX>;
+  // shared pattern bins: one set per warp, or 8 sets shared by the warps when the tables
+  // leave no room for more (the 6,144 shape)
+  constexpr int HC = DMAX == (1 << D_LOG2) ? WARPS : 8;
+  constexpr int T = TT::T, SH = 32 - TT::T_LOG2;
+  constexpr uint32_t RM = (1u << SH) - 1u, KM = (1u << D_LOG2) - 1u;
+  constexpr int NT = WARPS * 32;
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  TT& t = *reinterpret_cast<TT*>(dyn_smem);
+  __shared__ uint32_t hist[HC][kBins];
+  __shared__ int32_t s_r;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int k = threadIdx.x; k < HC * kBins; k += NT) (&hist[0][0])[k] = 0;
+  const int32_t n = *list.n;
+  RunHist rh;
+  unsigned long long probes = 0, gathers = 0, outs = 0, since_flush = 0;
+  int32_t cur = 0;   // member whose bins the shared histograms hold
+  auto block_flush = [&]() {
+    rh.flush(hist[w % HC]);
+    __syncthreads();
+    for (int k = threadIdx.x; k < kBins; k += NT) {
+      unsigned long long x = 0;
+      for (int ww = 0; ww < HC; ++ww) {
+        x += hist[ww][k];
+        hist[ww][k] = 0;
+      }
+      if (x) atomicAdd(&hist_out[(size_t)cur * kBins + k], x);
+    }
+    __syncthreads();
+  };
+
+  while (true) {
+    __syncthreads();
+    if (threadIdx.x == 0) s_r = atomicAdd(counter, 1);
+    __syncthreads();
+    const int32_t r = s_r;
+    if (r >= n) break;
+    const int32_t u = list.get(r);
+    const int32_t m = member_of(g, u);   // the same on every thread
+    if (m != cur || since_flush > (1ull << 30)) {   // 32-bit bins stay far from overflow
+      block_flush();
+      cur = m;
+      since_flush = 0;
+    }
+    const int32_t du = o.dplus[u];
+    const int64_t bu = o.row_ptr[u];
+    const int64_t eb = g.e_ptr[u];
+    const int32_t szu = (int32_t)(g.e_ptr[u + 1] - eb);
+    {   // both cuckoo tables to empty, 16 bytes per store
+      uint4* c = reinterpret_cast<uint4*>(t.c1);
+      for (int s = threadIdx.x; s < 2 * T / 4; s += NT) c[s] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    }
+    if (threadIdx.x == 0) t.nstash = 0;
+    if (w == 0) {   // E_y ranges of the vertices of e_u and their prefix sums
+      int64_t yb = 0, len = 0;
+      if (lane < szu) {
+        const int32_t y = __ldg(g.e_idx + eb + lane);
+        yb = __ldg(g.v_ptr + y);
+        len = __ldg(g.v_ptr + y + 1) - yb;
+      }
+      int64_t incl = len;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int64_t o2 = __shfl_up_sync(kFull, incl, d);
+        if (lane >= d) incl += o2;
+      }
+      t.ylen[lane] = len;
+      t.yincl[lane] = incl;
+      t.ybeg[lane] = yb;
+    }
+    __syncthreads();
+    // 1. out(u) into the cuckoo set; out-degrees into kpre[k + 1] for the prefix sum
+    for (int k = threadIdx.x; k < du; k += NT) {
+      int32_t x, om;
+      get_entry<PACKED>(o, bu + k, x, om);
+      uint32_t key = (uint32_t)x, kk = (uint32_t)k;
+      bool second = false, placed = false;
+      for (int tries = 0; tries < kCuckooTries; ++tries) {
+        const uint32_t pa = key * (second ? kCuckooA2 : kCuckooA1);
+        const uint32_t slot = pa >> SH;
+        uint32_t* c = second ? t.c2 : t.c1;
+        const uint32_t e = atomicExch(&c[slot], ((pa & RM) << D_LOG2) | kk);
+        if (e == ~0u) {
+          placed = true;
+          break;
+        }
+        // the evicted key sat at `slot` of this table: rebuild it from slot and remainder
+        key = ((slot << SH) | (e >> D_LOG2)) * (second ? kCuckooA2Inv : kCuckooA1Inv);
+        kk = e & KM;
+        second = !second;
+      }
+      if (!placed) {
+        const int at = atomicAdd(&t.nstash, 1);
+        if (at < kStash) {
+          t.skey[at] = (int32_t)key;
+          t.sidx[at] = (int32_t)kk;
+        }
+      }
+      t.kbeg[k] = __ldg(o.row_ptr + x);
+      t.kpre[k + 1] = __ldg(o.dplus + x);
+      t.ksz[k] = (uint16_t)__ldg(g.esize + x);
+      t.kmask[k] = 0;
+    }
+    __syncthreads();
+    const int nst = t.nstash;   // read after a barrier: uniform
+    if (nst > kStash || handover) {   // the global-table teams take u
+      if (threadIdx.x == 0) over.put(u);
+      continue;
+    }
+    // 2. Omega_ux masks over the flat E_y range; prefix of the out-degrees (warp 0)
+    {
+      const int64_t total = t.yincl[31];
+      if (threadIdx.x == 0) gathers += (unsigned long long)total;
+      for (int64_t f = threadIdx.x; f < total; f += NT) {
+        int lo = 0, hi = 31;
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (t.yincl[mid] > f) hi = mid; else lo = mid + 1;
+        }
+        const int p = lo;
+        const int32_t x = __ldg(g.v_idx + t.ybeg[p] + (f - (t.yincl[p] - t.ylen[p])));
+        const int k = block_find(t, x, nst);
+        if (k >= 0) atomicOr(&t.kmask[k], 1u << p);
+      }
+    }
+    if (w == 0) {   // in place: kpre[k + 1] holds the out-degree of out-neighbour k
+      int32_t run = 0;
+      for (int k0 = 0; k0 < du; k0 += 32) {
+        const int k = k0 + lane;
+        const int32_t c = k < du ? t.kpre[k + 1] : 0;
+        int32_t incl = c;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const int32_t o2 = __shfl_up_sync(kFull, incl, d);
+          if (lane >= d) incl += o2;
+        }
+        if (k < du) t.kpre[k + 1] = run + incl;
+        run += __shfl_sync(kFull, incl, 31);
+      }
+      if (lane == 0) t.kpre[0] = 0;
+    }
+    __syncthreads();
+    // |e_x| -> |e_x| - omega_ux, the part of e_x outside e_u
+    for (int k = threadIdx.x; k < du; k += NT) t.ksz[k] = (uint16_t)(t.ksz[k] - __popc(t.kmask[k]));
+    __syncthreads();
+    const uint32_t fu = full_mask(szu);
+    const int32_t F = t.kpre[du];
+    since_flush += (unsigned long long)F;   // the same on every thread
+    if (threadIdx.x == 0) {
+      probes += (unsigned long long)F;
+      outs += (unsigned long long)du;
+    }
+    // 3. closure: warp w walks the flat slice [F*w/WARPS, F*(w+1)/WARPS)
+    const int32_t f_lo = (int32_t)((int64_t)F * w / WARPS), f_hi = (int32_t)((int64_t)F * (w + 1) / WARPS);
+    if (nst == 0)
+      block_walk<D_LOG2, WARPS, PACKED, DMAX, false>(t, o, u, du, f_lo, f_hi, nst, fu, hist[w % HC],
+                                                     rh, lane, w);
+    else
+      block_walk<D_LOG2, WARPS, PACKED, DMAX, true>(t, o, u, du, f_lo, f_hi, nst, fu, hist[w % HC],
+                                                    rh, lane, w);
+  }
+  block_flush();
+  if (threadIdx.x == 0) {
+    atomicAdd(&work[0], probes);
+    atomicAdd(&work[1], gathers);
+    atomicAdd(&work[2], outs);
+  }
+}
+
+// ------------------------------------------------------------------ block per u (wide)
+// Any |e_u| (masks of `words` 32-bit words) and any out-degree; tables in global scratch.
+
+// Per block: out(u) as a two-table cuckoo set coded by quotient like the block teams'
 // (2^(dl+1) slots per table for du <= 2^dl), a stash with room for every key (these
 // teams hand nothing over), and per out-neighbour arrays (Omega_ux of `words` words,
 // |e_x|, list length and start).  Only the slots and the du rows of masks in use are
@@ -529,8 +895,7 @@ __device__ __forceinline__ int wide_find(const WideScratch& t, int32_t x, int dl
 
 template <bool PACKED>
 __global__ void __launch_bounds__(kWideThreads, kWideBlocksPerSm)
-    k_close_wide(DevGraph g, Oriented o, const int32_t* __restrict__ list,
-                 const int32_t* __restrict__ n_p, int64_t cap_max, int64_t words_max,
+    k_close_wide(DevGraph g, Oriented o, OwnerList list, int64_t cap_max, int64_t words_max,
                  int64_t dmax, char* __restrict__ scratch, unsigned long long* __restrict__ hist_out,
                  unsigned long long* __restrict__ work, int32_t* __restrict__ counter) {
   __shared__ uint32_t hist[kHistCopies][kBins];
@@ -545,7 +910,7 @@ __global__ void __launch_bounds__(kWideThreads, kWideBlocksPerSm)
   WideScratch t = wide_carve(scratch + wide_block_bytes(cap_max, words_max, dmax) * blockIdx.x,
                              cap_max, words_max, dmax);
   for (int k = threadIdx.x; k < kHistCopies * kBins; k += blockDim.x) (&hist[0][0])[k] = 0;
-  const int32_t n = *n_p;
+  const int32_t n = *list.n;
   uint32_t* my_hist = hist[lane & (kHistCopies - 1)];
   unsigned long long probes = 0, gathers = 0, outs = 0;
   int32_t cur = 0;   // member whose bins the shared histograms hold
@@ -569,7 +934,7 @@ __global__ void __launch_bounds__(kWideThreads, kWideBlocksPerSm)
     __syncthreads();
     const int32_t r = s_r;
     if (r >= n) break;
-    const int32_t u = list[r];
+    const int32_t u = list.get(r);
     const int32_t m = member_of(g, u);   // the same on every thread
     if (m != cur || s_since > (1ull << 28)) {   // s_since is read after a barrier: uniform
       block_flush();
@@ -739,8 +1104,7 @@ __device__ __forceinline__ int wide_find_l2(const WideScratch& t, int32_t x, int
 
 template <bool PACKED>
 __global__ void __launch_bounds__(kClusterThreads, 1)
-    k_close_cluster(DevGraph g, Oriented o, const int32_t* __restrict__ list,
-                    const int32_t* __restrict__ n_p, int64_t cap_max, int64_t words_max,
+    k_close_cluster(DevGraph g, Oriented o, OwnerList list, int64_t cap_max, int64_t words_max,
                     int64_t dmax, char* __restrict__ scratch,
                     unsigned long long* __restrict__ hist_out, unsigned long long* __restrict__ work,
                     int32_t* __restrict__ counter) {
@@ -765,7 +1129,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1)
                                            (size_t)(blockIdx.x / csize),
                              cap_max, words_max, dmax);
   for (int k = threadIdx.x; k < kHistCopies * kBins; k += kClusterThreads) (&hist[0][0])[k] = 0;
-  const int32_t n = *n_p;
+  const int32_t n = *list.n;
   uint32_t* my_hist = hist[lane & (kHistCopies - 1)];
   RunHist rh;
   unsigned long long probes = 0, gathers = 0, outs = 0;
@@ -794,7 +1158,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1)
       cluster.sync();   // rank 0's shared memory stays until every block has read it
       break;
     }
-    const int32_t u = list[r];
+    const int32_t u = list.get(r);
     const int32_t m = member_of(g, u);
     if (m != cur || s_since > (1ull << 28)) {   // read after a barrier: uniform in the block
       block_flush();
@@ -1010,14 +1374,18 @@ __device__ __forceinline__ int list_of(int label, int32_t d, int32_t sz, int32_t
   if (label < 0) return -1;
   if (rule.all_wide) return kListWide;
   const int c = bit_class_of(d, sz, osum, nv);
+  if (c < 0) return label;
+  const bool hash = c == kBitClasses - 1 && nv > kBitMapVertices;
+  // (an owner that fills the hash has read most of its vertices for nothing)
+  if (hash && osum + sz > kBitHashEntries) return label;
   const int64_t ratio = c < 3 ? kWalkRatio0 : (c == 3 ? kWalkRatio3 : kWalkRatio4);
-  if (label <= 2 && (c < 0 || dsum < ratio * osum)) return label;
+  if (label <= 2 && dsum < ratio * osum) return label;
   // (the last class with a hash dictionary loses to the global-table blocks there: 2.3
   // against 1.2 ms on the batch members' hyperedges of more than 32 vertices)
-  if (c >= 0 && !(c == kBitClasses - 1 && label == kWideBucket &&
-                  dsum < kWalkRatio4 * (int64_t)osum && nv > kBitDirectVertices))
-    return kListBits + c;
-  return label == kClusterBucket ? kListCluster : (label == kWideBucket ? kListWide : kListOver);
+  if (c == kBitClasses - 1 && label == kWideBucket && dsum < kWalkRatio4 * (int64_t)osum &&
+      nv > kBitDirectVertices)
+    return label;
+  return kListBits + c;
 }
 
 // Each block takes kBucketRowsPerBlock hyperedges: places within the block by shared atomics
@@ -1048,12 +1416,9 @@ __global__ void __launch_bounds__(kBucketThreads)
       if (bk[q] >= 0) {
         at[q] = atomicAdd(&s_cnt[bk[q]], 1);
         atomicAdd(&s_label[label], 1);
-        mx[2] = max(mx[2], d);
-        mx[3] = max(mx[3], sz);
-        if (bk[q] == kListWide || bk[q] == kListCluster) {
-          mx[0] = max(mx[0], d);
-          mx[1] = max(mx[1], sz);
-        }
+        const int w = label >= kWideBucket ? 0 : 2;   // (a bit-row team may return u to it)
+        mx[w] = max(mx[w], d);
+        mx[w + 1] = max(mx[w + 1], sz);
         if (bk[q] == kListBits + kBitClasses - 1) {
           mx[4] = max(mx[4], os);
           mx[5] = max(mx[5], d);
@@ -1069,7 +1434,7 @@ __global__ void __launch_bounds__(kBucketThreads)
   __syncthreads();
   if (threadIdx.x < kLists) {
     const int32_t n = s_cnt[threadIdx.x];
-    s_base[threadIdx.x] = n ? atomicAdd(&b.count[threadIdx.x], n) : 0;
+    s_base[threadIdx.x] = n ? atomicAdd(b.list[threadIdx.x].n, n) : 0;
   }
   if (threadIdx.x >= 32 && threadIdx.x < 32 + kCloseBuckets) {
     const int k = threadIdx.x - 32;
@@ -1083,15 +1448,13 @@ __global__ void __launch_bounds__(kBucketThreads)
 #pragma unroll
   for (int q = 0; q < kBucketRowsPerThread; ++q)
     if (bk[q] >= 0)
-      b.lists[bk[q]][s_base[bk[q]] + at[q]] = (int32_t)((int64_t)blockIdx.x * kBucketRowsPerBlock +
-                                                        q * kBucketThreads + threadIdx.x);
+      b.list[bk[q]].at[(int64_t)(s_base[bk[q]] + at[q]) * b.list[bk[q]].step] =
+          (int32_t)((int64_t)blockIdx.x * kBucketRowsPerBlock + q * kBucketThreads + threadIdx.x);
 }
 
 template <int D_LOG2, int WARPS, bool PACKED, bool OFF32>
-void launch_warp_t(const DevGraph& g, const Oriented& o, const int32_t* list, int32_t n,
-                   const int32_t* n_p, unsigned long long* hist, unsigned long long* work,
-                   int32_t* counter, int32_t* overflow, int32_t* n_overflow, int handover,
-                   cudaStream_t s, int nsm) {
+void launch_warp_t(const CloseRun& r, const OwnerList& list, int32_t n,
+                   unsigned long long* work, int32_t* counter) {
   auto kern = k_close_warp<D_LOG2, WARPS, PACKED, OFF32>;
   const int smem = (int)(WARPS * sizeof(WarpTables<D_LOG2, PACKED, OFF32>));
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -1099,30 +1462,48 @@ void launch_warp_t(const DevGraph& g, const Oriented& o, const int32_t* list, in
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, WARPS * 32, smem);
   if (per_sm < 1) per_sm = 1;
   int blocks = (n + WARPS - 1) / WARPS;
-  if (blocks > per_sm * nsm) blocks = per_sm * nsm;
+  if (blocks > per_sm * r.nsm) blocks = per_sm * r.nsm;
   note_launch();
-  kern<<<blocks, WARPS * 32, smem, s>>>(g, o, list, n_p, hist, work, counter, overflow,
-                                         n_overflow, handover);
+  kern<<<blocks, WARPS * 32, smem, r.s>>>(r.g, r.o, list, r.hist, work, counter, r.over,
+                                           r.handover);
 }
 
 template <int D_LOG2, int WARPS>
-void launch_warp(const DevGraph& g, const Oriented& o, int packed, const int32_t* list, int32_t n,
-                 const int32_t* n_p, unsigned long long* hist, unsigned long long* work,
-                 int32_t* counter, int32_t* overflow, int32_t* n_overflow, int handover,
-                 cudaStream_t s, int nsm) {
-  const bool off32 = o.slots > 0 && o.slots < (int64_t(1) << 32);
-  if (packed && off32)
-    launch_warp_t<D_LOG2, WARPS, true, true>(g, o, list, n, n_p, hist, work, counter, overflow,
-                                             n_overflow, handover, s, nsm);
-  else if (packed)
-    launch_warp_t<D_LOG2, WARPS, true, false>(g, o, list, n, n_p, hist, work, counter, overflow,
-                                              n_overflow, handover, s, nsm);
-  else if (off32)
-    launch_warp_t<D_LOG2, WARPS, false, true>(g, o, list, n, n_p, hist, work, counter, overflow,
-                                              n_overflow, handover, s, nsm);
-  else
-    launch_warp_t<D_LOG2, WARPS, false, false>(g, o, list, n, n_p, hist, work, counter,
-                                               overflow, n_overflow, handover, s, nsm);
+void launch_warp(const CloseRun& r, const OwnerList& list, int32_t n, unsigned long long* work,
+                 int32_t* counter) {
+  const bool off32 = r.o.slots > 0 && r.o.slots < (int64_t(1) << 32);
+  if (r.packed && off32) launch_warp_t<D_LOG2, WARPS, true, true>(r, list, n, work, counter);
+  else if (r.packed) launch_warp_t<D_LOG2, WARPS, true, false>(r, list, n, work, counter);
+  else if (off32) launch_warp_t<D_LOG2, WARPS, false, true>(r, list, n, work, counter);
+  else launch_warp_t<D_LOG2, WARPS, false, false>(r, list, n, work, counter);
+}
+
+template <int D_LOG2, int WARPS, bool PACKED, int DMAX = (1 << D_LOG2)>
+void launch_block_t(const CloseRun& r, const OwnerList& list, int32_t n,
+                    unsigned long long* work, int32_t* counter) {
+  auto kern = k_close_block<D_LOG2, WARPS, PACKED, DMAX>;
+  const int smem = (int)sizeof(BlockTables<D_LOG2, WARPS, PACKED, DMAX>);
+  // the tables plus the kernel's static bins (one set per warp, or 8) and fetch slot fit
+  // the 232,448 bytes of shared memory a block may use
+  static_assert(sizeof(BlockTables<D_LOG2, WARPS, PACKED, DMAX>) +
+                        sizeof(uint32_t) * kBins * (DMAX == (1 << D_LOG2) ? WARPS : 8) + 16 <=
+                    232448,
+                "block-team shared memory");
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  int per_sm = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, WARPS * 32, smem);
+  if (per_sm < 1) per_sm = 1;
+  const int blocks = n < per_sm * r.nsm ? n : per_sm * r.nsm;
+  note_launch();
+  kern<<<blocks, WARPS * 32, smem, r.s>>>(r.g, r.o, list, r.hist, work, counter, r.over,
+                                           r.handover);
+}
+
+template <int D_LOG2>
+void launch_block(const CloseRun& r, const OwnerList& list, int32_t n, unsigned long long* work,
+                  int32_t* counter) {
+  if (r.packed) launch_block_t<D_LOG2, kBlockWarps, true>(r, list, n, work, counter);
+  else launch_block_t<D_LOG2, kBlockWarpsUnpacked, false>(r, list, n, work, counter);
 }
 
 }  // namespace
@@ -1140,24 +1521,18 @@ size_t close_wide_scratch_bytes(int64_t cap, int64_t words, int64_t dmax, int ns
   return wide_block_bytes(cap, words, dmax) * (size_t)(nsm * kWideBlocksPerSm);
 }
 
-cudaError_t launch_close(int list_id, const DevGraph& g, const Oriented& o, int packed,
-                  const int32_t* list, int32_t n, const int32_t* n_p, int64_t wide_cap,
-                  int64_t wide_words, int64_t wide_dmax, void* scratch, unsigned long long* hist,
-                  unsigned long long* work, int32_t* counter, int32_t* overflow,
-                  int32_t* n_overflow, int handover, cudaStream_t s, int nsm) {
+cudaError_t launch_close(int list_id, const CloseRun& r, const OwnerList& list, int32_t n,
+                         const WideSpace& w, unsigned long long* work, int32_t* counter) {
   if (n <= 0) return cudaSuccess;
   switch (list_id) {
-    case 0:
-      launch_warp<6, 8>(g, o, packed, list, n, n_p, hist, work, counter, overflow, n_overflow,
-                        handover, s, nsm);
-      break;
-    case 1:
-      launch_warp<7, 6>(g, o, packed, list, n, n_p, hist, work, counter, overflow, n_overflow,
-                        handover, s, nsm);
-      break;
-    case 2:
-      launch_warp<8, 4>(g, o, packed, list, n, n_p, hist, work, counter, overflow, n_overflow,
-                        handover, s, nsm);
+    case 0: launch_warp<6, 8>(r, list, n, work, counter); break;
+    case 1: launch_warp<7, 6>(r, list, n, work, counter); break;
+    case 2: launch_warp<8, 4>(r, list, n, work, counter); break;
+    case 3: launch_block<10>(r, list, n, work, counter); break;
+    case 4: launch_block<11>(r, list, n, work, counter); break;
+    case 5:   // the packed layout's shape reaches out-degree 6,144 (13-bit indices)
+      if (r.packed) launch_block_t<13, kBlockWarps, true, kBlockMaxPacked>(r, list, n, work, counter);
+      else launch_block_t<12, kBlockWarpsUnpacked, false>(r, list, n, work, counter);
       break;
     case kListCluster: {
       // clusters of kWideCluster blocks, as many as can be resident at once
@@ -1169,35 +1544,30 @@ cudaError_t launch_close(int list_id, const DevGraph& g, const Oriented& o, int 
       attr[0].val.clusterDim.z = 1;
       cfg.blockDim = dim3(kClusterThreads);
       cfg.dynamicSmemBytes = 0;
-      cfg.stream = s;
+      cfg.stream = r.s;
       cfg.attrs = attr;
       cfg.numAttrs = 1;
-      auto kern = packed ? k_close_cluster<true> : k_close_cluster<false>;
+      auto kern = r.packed ? k_close_cluster<true> : k_close_cluster<false>;
       int clusters = 0;
-      cfg.gridDim = dim3((unsigned)(nsm / kWideCluster * kWideCluster));
+      cfg.gridDim = dim3((unsigned)(r.nsm / kWideCluster * kWideCluster));
       if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters < 1) {
         cudaGetLastError();
-        clusters = nsm / kWideCluster;
+        clusters = r.nsm / kWideCluster;
       }
       if (clusters > n) clusters = n;
       if (clusters < 1) clusters = 1;
       cfg.gridDim = dim3((unsigned)(clusters * kWideCluster));
       note_launch();
-      cudaLaunchKernelEx(&cfg, kern, g, o, list, n_p, wide_cap, wide_words, wide_dmax,
-                         (char*)scratch, hist, work, counter);
+      cudaLaunchKernelEx(&cfg, kern, r.g, r.o, list, w.cap, w.words, w.dmax, (char*)w.scratch,
+                         r.hist, work, counter);
       break;
     }
     default: {
-      int blocks = n < nsm * kWideBlocksPerSm ? n : nsm * kWideBlocksPerSm;
+      const int blocks = n < r.nsm * kWideBlocksPerSm ? n : r.nsm * kWideBlocksPerSm;
+      auto kern = r.packed ? k_close_wide<true> : k_close_wide<false>;
       note_launch();
-      if (packed)
-        k_close_wide<true><<<blocks, kWideThreads, 0, s>>>(g, o, list, n_p, wide_cap, wide_words,
-                                                           wide_dmax, (char*)scratch, hist, work,
-                                                           counter);
-      else
-        k_close_wide<false><<<blocks, kWideThreads, 0, s>>>(g, o, list, n_p, wide_cap, wide_words,
-                                                            wide_dmax, (char*)scratch, hist, work,
-                                                            counter);
+      kern<<<blocks, kWideThreads, 0, r.s>>>(r.g, r.o, list, w.cap, w.words, w.dmax,
+                                             (char*)w.scratch, r.hist, work, counter);
     }
   }
   return cudaGetLastError();
