@@ -288,6 +288,7 @@ struct OwnerList {
 #endif
 };
 constexpr int kWalkRatio0 = 8, kWalkRatio3 = 40, kWalkRatio4 = 80;   // see list_of in k_close.cu
+constexpr int kWalkRatioWide = 8;
 constexpr int kBitMaxOut = 8192;             // bit rows: out-degree, column-list entries
 constexpr int kBitMaxEntries = 1 << 22;
 // Direct vertex map up to kBitDirectVertices; its bit maps alone in shared memory up to
@@ -306,13 +307,16 @@ constexpr int kBitSmem = 232448 - 2048;      // dynamic shared memory a block ma
 constexpr int kBitPlanes = 16;               // digits of a shared count (<= 65,535)
 constexpr int kBitLargeSlots = 14;           // log2 slots of the last class's hash dictionary
 
-// Shared memory of the last class before its columns: digits and flags, e_u's columns
-// twice, the rows, and the vertex dictionary.
-__host__ __device__ inline int64_t bit_large_bytes(int64_t du, int64_t szu, int64_t nv) {
+// Shared memory of the last class: digits and flags, e_u's columns twice and the rows, then the
+// vertex dictionary, whose place the columns take later.
+__host__ __device__ inline int64_t bit_rows_bytes(int64_t du, int64_t szu) {
   const int64_t W = (du + 31) / 32;
-  return 4 * (kBitPlanes + 1) * W + 8 * szu * W + 23 * du +
+  return 4 * (kBitPlanes + 1) * W + 8 * szu * W + 23 * du + 256;
+}
+__host__ __device__ inline int64_t bit_large_bytes(int64_t du, int64_t szu, int64_t nv) {
+  return bit_rows_bytes(du, szu) +
          (nv <= kBitMapVertices ? 8 * ((nv + 31) / 32) + (nv <= kBitDirectVertices ? 2 * nv : 0)
-                                : 6ll << kBitLargeSlots) + 256;
+                                : 6ll << kBitLargeSlots);
 }
 
 // Global scratch of a block for the columns by vertex.

@@ -1355,18 +1355,31 @@ __global__ void __launch_bounds__(kClusterThreads, 1)
 
 // ------------------------------------------------------------------ bucketing
 
-// List of u (-1 when u closes nothing).  An owner the warp teams can take (labels 0-2) walks
-// its out-lists when its neighbourhood is sparse for the bit-row team it would need: dsum,
+// List of u (-1 when u closes nothing).  u goes to the walking team of its label when no
+// bit-row team holds it or when its neighbourhood is sparse for the one it would need: dsum,
 // the degrees of its out-neighbours, stands for the entries of their out-lists that a walk
 // looks up (these are about a quarter of it), osum for the vertices the bit rows lay out.
-// Measured, closure ms of (co-authorship shape, 30,000 hyperedges of its kind, 64 batch
-// members); 8.03, 0.66, 52.0 with every such owner walked:
+//
+// Against warp teams, closure ms of (co-authorship shape, 30,000 hyperedges of its kind, 64
+// batch members); 8.03, 0.66, 52.0 with every such owner walked:
 //   class 3 (16 warps) by bit rows from dsum / osum = 0: 5.99, 0.53, 51.4; 40: 5.99, 0.53,
 //     50.7; 45: 6.07, 0.53, 49.3; 50: 6.17, 0.68, 48.8; 80: 6.10, 0.66, 49.1 (a few long walks
 //     are the tail of the smaller ones);
 //   class 4 (32 warps) from 0: 62.7 on the members; 50: 53.0; 60: 48.9; 80: 48.8;
 //   classes 0-2 from 0, 4, 8, 12: within 0.02 of each other everywhere; 20: 6.12, 0.68, 49.1;
 //     40: 6.34, 0.68, 48.6.  Below 8 there is next to nothing to look up.
+// Against block teams the same lines hold.  The last class, ms of (20,011 hyperedges of up to
+// 600 vertices over 60,000, 60,000 of a larger mean size over as many), from 0: 12.1, 1,040;
+// 40: 10.8, 1,042; 60: 10.8, 968; 80: 10.8, 967; 100: 10.8, 970; the ratio of the tag shapes is
+// above 110, and there block teams need three times as long.  With the hash dictionary (100,000
+// hyperedges of up to 600 over 300,000 vertices) from 0: 151; 40: 125; 60: 83.7; 80: 83.4.
+// Against the global-table teams (|e_u| > 32 or the largest out-degrees): a pair costs bit rows
+// a step per vertex of e_u and v, so large hyperedges over few others lose.  From 0 / 5 / 7 /
+// 14 / 40 / 60: 1,500 hyperedges of 300-600 vertices 31.3 / 17.0 / 18.2 / 16.3 / 16.7 / 16.2,
+// 2,000 of 100-200 11.7 / 11.8 / 11.5 / 13.3 / 13.2 / 13.0, 3,000 of 40-80 9.4 / 9.3 / 9.3 /
+// 9.4 / 23.2 / 22.7, 300 of 1,000-4,000 7.0 / 2.7 / 2.3 / 2.5 / 2.3 / 2.3.  Where the columns (at
+// most osum / 2, and |V|) may not fit, trying costs up to a third of the walk, so that takes the
+// ratio of the last class.
 // On the uniform and tag shapes the ratio is 110-220 and bit rows take 0.5 against 2.2 ms
 // (1,000 vertices, 2,000 hyperedges).
 __device__ __forceinline__ int list_of(int label, int32_t d, int32_t sz, int32_t osum,
@@ -1375,17 +1388,15 @@ __device__ __forceinline__ int list_of(int label, int32_t d, int32_t sz, int32_t
   if (rule.all_wide) return kListWide;
   const int c = bit_class_of(d, sz, osum, nv);
   if (c < 0) return label;
-  const bool hash = c == kBitClasses - 1 && nv > kBitMapVertices;
-  // (an owner that fills the hash has read most of its vertices for nothing)
-  if (hash && osum + sz > kBitHashEntries) return label;
-  const int64_t ratio = c < 3 ? kWalkRatio0 : (c == 3 ? kWalkRatio3 : kWalkRatio4);
-  if (label <= 2 && dsum < ratio * osum) return label;
-  // (the last class with a hash dictionary loses to the global-table blocks there: 2.3
-  // against 1.2 ms on the batch members' hyperedges of more than 32 vertices)
-  if (c == kBitClasses - 1 && label == kWideBucket && dsum < kWalkRatio4 * (int64_t)osum &&
-      nv > kBitDirectVertices)
-    return label;
-  return kListBits + c;
+  int64_t ratio = c < 3 ? kWalkRatio0 : (c == 3 ? kWalkRatio3 : kWalkRatio4);
+  if (c == kBitClasses - 1 && nv > kBitMapVertices) {
+    // (an owner that fills the hash has read most of its vertices for nothing)
+    if (osum + sz > kBitHashEntries) return label;
+  } else if (label >= kWideBucket) {
+    const int64_t words = (kBitSmem - bit_rows_bytes(d, sz)) / 4;
+    if ((nv < osum / 2 ? nv : osum / 2) <= words + words / 4) ratio = kWalkRatioWide;
+  }
+  return dsum < ratio * osum ? label : kListBits + c;
 }
 
 // Each block takes kBucketRowsPerBlock hyperedges: places within the block by shared atomics

@@ -46,3 +46,45 @@ def test_out_degrees_beyond_the_bit_rows(hglib):
     assert st["max_out_deg"] > 4000 and st["close"]["bucket_teams"][6] == 0
     for k in ("probes", "gathers", "out_entries"):
         assert st["close"][k] == ws["close"][k], k
+
+
+def closed_by(hg, nv, e_ptr, e_idx):
+    """(counts, masks, names of the closure kernels that ran)"""
+    import torch
+
+    g = hg.hg_load_csr(nv, len(e_ptr) - 1, e_ptr, e_idx, stream=torch.cuda.Stream().cuda_stream)
+    try:
+        hg.hg_set_timing(g, True)
+        hg.hg_build_wedges(g)
+        counts = hg.hg_count_patterns(g)
+        return counts, {k for k in hg.hg_kernel_times(g) if k.startswith("close_")}
+    finally:
+        hg.hg_free(g)
+
+
+@pytest.mark.parametrize("nv,ne,lo,hi,shift,bits", [
+    (3000, 120, 400, 800, 0, False),      # |e_u| of hundreds over few others: walked
+    (300, 420, 33, 38, 50_000, True),     # beyond the direct map: bit rows all the same
+    (300, 420, 33, 38, 300_000, False),   # the hash dictionary is for dense ones alone
+])
+def test_owners_of_more_than_32_vertices(hglib, nv, ne, lo, hi, shift, bits):
+    edges = random_edges(nv, ne, lo, hi, ne)
+    e_ptr, e_idx = csr_of([[v + shift for v in e] for e in edges])
+    check_against_oracle(hglib, nv + shift, e_ptr, e_idx)
+    _, kernels = closed_by(hglib, nv + shift, e_ptr, e_idx)
+    assert kernels >= ({"close_bits_large"} if bits else {"close_wide"})
+    if not bits:
+        assert "close_bits_large" not in kernels
+
+
+def test_sparse_owners_with_long_neighbours_go_to_the_block_teams(hglib):
+    # 300 small hyperedges and 60 of 300-500 vertices meet in vertex 0: the small ones rank
+    # lowest, have out-degrees above 256, and their neighbours' vertices are many and private
+    rng = np.random.default_rng(4)
+    edges = {(0, 1 + k, 301 + k) for k in range(300)}
+    edges |= {tuple([0] + (1000 + np.sort(rng.choice(40_000, int(n), replace=False))).tolist())
+              for n in rng.integers(300, 500, 60)}
+    e_ptr, e_idx = csr_of([list(e) for e in sorted(edges)])
+    check_against_oracle(hglib, 41_000, e_ptr, e_idx)
+    _, kernels = closed_by(hglib, 41_000, e_ptr, e_idx)
+    assert "close_block2048" in kernels
