@@ -217,7 +217,13 @@ __device__ int triple_common(const int32_t* a, int na, const int32_t* b, int nb,
 constexpr int kCacheEntries = 384;   // searched rows up to this long go to shared memory
 constexpr int kCommonMax = 64;       // e_i cap e_j up to this large goes to shared memory
 constexpr int kHitQueue = 64;        // a round of 32 candidates plus a partial one
-constexpr int kScanMax = 32;         // e_k up to this large is scanned, not searched
+// e_k up to this large is scanned, not searched.  A scan waits less, a search reads less: on
+// 500,000 co-authorship hyperedges (rows from memory) Algorithm 6 takes 3.82 ms for 2 million
+// draws with 32, 3.95 with 16, 3.90 with 8.  Algorithm 7 walks whole rows, whose hits are more
+// and mostly cached: 500,000 draws on 10,000 tag-shaped hyperedges take 37.9 ms with 32, 35.0
+// with 16, 33.2 with 8 (36.7 before hits were queued, by searches alone), on the co-authorship
+// shape 2.43, 2.49, 2.46 (2.95).
+constexpr int kScanMax = 32, kScanMaxAdv = 8;
 
 template <bool PACKED>
 struct WarpCache {
@@ -360,13 +366,13 @@ __device__ __forceinline__ bool stage_common(WarpCache<PACKED>& c, const int32_t
 }
 
 // g = |e_i cap e_j cap e_k|
-template <bool PACKED>
+template <bool PACKED, int SCAN>
 __device__ __forceinline__ int common3(const WarpCache<PACKED>& c, bool staged, int wij,
                                        const int32_t* ei, int szi, const int32_t* ej, int szj,
                                        const int32_t* ek, int szk, ReadCount& rc) {
   if (staged) {
     int gg = 0;
-    if (szk <= kScanMax) {
+    if (szk <= SCAN) {
       for (int p = 0; p < szk; p += 8) {   // eight independent loads
         int32_t x[8];
 #pragma unroll
@@ -530,7 +536,7 @@ __global__ void __launch_bounds__(kSampleWarps * 32)
           if (!valid) return;
           int szk;
           const int32_t* ek = edge_of(g, k, szk);
-          const int gg = common3<PACKED>(cw, staged, wij, ei, szi, ej, szj, ek, szk, rc);
+          const int gg = common3<PACKED, kScanMax>(cw, staged, wij, ei, szi, ej, szj, ek, szk, rc);
           atomicAdd(&hist[w][lut[region_bits7(szi, szj, szk, wij, wik, wjk, gg)]], 1u);
         });
   }
@@ -611,11 +617,16 @@ struct AdvSet {
 
 __device__ __forceinline__ int wedge_type(int om, int sa, int sb) { return om == min(sa, sb); }
 
+// Blocks per SM that the registers are held to: the searches of whole rows wait on one load
+// after another, and 63 registers left room for 4 (500,000 draws on the co-authorship shape 2.61
+// ms, 2.43 with 5; on 10,000 tag-shaped hyperedges 39.0 and 37.9).
+constexpr int kAdvBlocks = 5;
+
 // One warp per draw of set `st`: the drawn (i, j), every k in N(i) cap N(j) (the shorter
 // row walked, the longer searched); the triangle counts when its class is st.cls and
 // (i, j) is its first hyperwedge of type st.type in O.  raw[0..23] += per-pattern counts.
 template <bool PACKED>
-__global__ void __launch_bounds__(kSampleWarps * 32)
+__global__ void __launch_bounds__(kSampleWarps * 32, kAdvBlocks)
     k_sample_adv(DevGraph g, AdvSet st, const int64_t* __restrict__ full_ptr, Oriented full,
                  uint64_t seed, uint64_t first, uint64_t num,
                  unsigned long long* __restrict__ raw) {
@@ -663,7 +674,7 @@ __global__ void __launch_bounds__(kSampleWarps * 32)
           const int wik = swap ? wb : wa, wjk = swap ? wa : wb;
           int szk;
           const int32_t* ek = edge_of(g, k, szk);
-          const int gg = common3<PACKED>(cw, staged, wij, ei, szi, ej, szj, ek, szk, rc);
+          const int gg = common3<PACKED, kScanMaxAdv>(cw, staged, wij, ei, szi, ej, szj, ek, szk, rc);
           const int pat = lut[region_bits7(szi, szj, szk, wij, wik, wjk, gg)];
           if (c_class_of[pat] != st.cls) return;
           // the triangle's hyperwedges in O, (a,b) < (a,c) < (b,c) for a < b < c; the
@@ -729,7 +740,7 @@ __global__ void __launch_bounds__(kSampleWarps * 32)
           if (valid && target != 0) {
             int szk;
             const int32_t* ek = edge_of(g, k, szk);
-            const int gg = common3<PACKED>(cw, staged, wij, ei, szi, ej, szj, ek, szk, rc);
+            const int gg = common3<PACKED, kScanMax>(cw, staged, wij, ei, szi, ej, szj, ek, szk, rc);
             hit = lut[region_bits7(szi, szj, szk, wij, wik, wjk, gg)] == target;
           }
           const unsigned bal = __ballot_sync(kFull, hit);
