@@ -183,6 +183,17 @@ void release(hg_graph* g, std::vector<Block>& owner) {
   owner.clear();
 }
 
+// One block of an owner, given back before the others.
+void release_one(hg_graph* g, std::vector<Block>& owner, void* p) {
+  for (size_t k = 0; k < owner.size(); ++k) {
+    if (owner[k].p != p) continue;
+    std::vector<Block> one{owner[k]};
+    owner.erase(owner.begin() + (int64_t)k);
+    release(g, one);
+    return;
+  }
+}
+
 hg_status cuda_status(cudaError_t e) { return e == cudaSuccess ? HG_OK : HG_ERR_CUDA; }
 
 #define HG_CUDA(call)                                        \
@@ -1151,14 +1162,20 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
   for (int k = 0; k < kLists; ++k) n[k] = h.list_count[k];
   // scratch of the global-table teams: out-degrees and |e_u| up to the two maxima
   auto wide_scratch = [&](unsigned long long dmax, unsigned long long smax, WideSpace* w) {
-    w->dmax = std::max<int64_t>((int64_t)dmax, 1);
-    w->words = std::max<int64_t>(((int64_t)smax + 31) / 32, 1);
-    while (w->cap < 2 * w->dmax) w->cap *= 2;
+    WideSpace need;
+    need.dmax = std::max<int64_t>((int64_t)dmax, 1);
+    need.words = std::max<int64_t>(((int64_t)smax + 31) / 32, 1);
+    while (need.cap < 2 * need.dmax) need.cap *= 2;
+    if (w->scratch) {   // of an earlier launch: kept when it is large enough
+      if (w->cap >= need.cap && w->words >= need.words && w->dmax >= need.dmax) return true;
+      release_one(g, g->count_blocks, w->scratch);
+    }
+    *w = need;
     w->scratch = dev_alloc(g, g->count_blocks,
                            close_wide_scratch_bytes(w->cap, w->words, w->dmax, g->nsm));
     return w->scratch != nullptr;
   };
-  WideSpace wide, over;
+  WideSpace wide;
   const int64_t slice_dmax = ((int64_t)h.close_max[5] + 15) / 16 * 16;
   const int64_t slice = bits_slice_bytes(slice_dmax, (int64_t)h.close_max[4], g->nv);
   const int slice_blocks = std::min(n[kListBits + kBitClasses - 1], g->nsm);
@@ -1185,12 +1202,11 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
   }
   // A walking team's list and what the bit-row teams gave back to it (`most`: an upper bound).
   auto walk = [&](int k, int64_t most) {
-    if (k >= kListWide && k <= kListCluster && !wide.scratch &&
+    if (k >= kListWide && k <= kListCluster &&
         !wide_scratch(h.close_max[0], h.close_max[1], &wide))
       return HG_ERR_OOM;
     t_begin(g, names[k]);
-    HG_CUDA(launch_close(k, run, cl.list[k], (int32_t)std::min<int64_t>(most, ne),
-                         k == kListOver ? over : wide,
+    HG_CUDA(launch_close(k, run, cl.list[k], (int32_t)std::min<int64_t>(most, ne), wide,
                          g->small->work[k == kListOver ? kWideBucket : k], g->small->counters + k));
     t_end(g);
     return HG_OK;
@@ -1207,7 +1223,9 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
   if (more) HG_TRY(sync_small(g, &h));
   const int32_t n_over = h.list_count[kListOver];
   if (n_over > 0) {
-    if (!wide_scratch(h.close_max[2], h.close_max[3], &over)) return HG_ERR_OOM;
+    // (the teams before are done: their scratch is reused or given back)
+    if (slices) release_one(g, g->count_blocks, slices);
+    if (!wide_scratch(h.close_max[2], h.close_max[3], &wide)) return HG_ERR_OOM;
     HG_TRY(walk(kListOver, n_over));
     HG_TRY(sync_small(g, &h));
   }

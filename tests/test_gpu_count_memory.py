@@ -1,0 +1,67 @@
+"""Device memory that a count holds at a time, seen through the allocator hooks."""
+import pytest
+
+from conftest import csr_of
+from test_gpu_bit_rows import random_edges
+
+pytestmark = pytest.mark.gpu
+
+
+class Counting:
+    """Hooks over torch's allocator that keep the bytes of every live block and the peak."""
+
+    def __init__(self, hg):
+        import torch
+
+        self.live, self.peak = {}, 0
+        self.on_change = None
+
+        def alloc(nbytes, stream, _ctx):
+            p = torch.cuda.caching_allocator_alloc(int(nbytes), torch.cuda.current_device(),
+                                                   int(stream or 0))
+            self.live[p] = int(nbytes)
+            self.peak = max(self.peak, sum(self.live.values()))
+            if self.on_change:
+                self.on_change(self.live)
+            return p
+
+        def free(p, _nbytes, _stream, _ctx):
+            self.live.pop(p)
+            torch.cuda.caching_allocator_delete(int(p))
+
+        self.hooks = (hg.hg._ALLOC_FN(alloc), hg.hg._FREE_FN(free))
+        hg.hg_set_allocator(*self.hooks)
+
+
+def test_one_scratch_of_the_global_table_teams_at_a_time(hglib):
+    # hyperedges of 60-70 vertices (global-table teams) and of 20-32 (handed over to the same
+    # teams by close_mode 2): the scratch of the second launch takes the place of the first's
+    import torch
+
+    edges = random_edges(400, 150, 60, 70, 1) + random_edges(400, 250, 20, 32, 2)
+    e_ptr, e_idx = csr_of(edges)
+    count = Counting(hglib)
+    try:
+        big = []
+        g = hglib.hg_load_csr(400, len(e_ptr) - 1, e_ptr, e_idx,
+                              stream=torch.cuda.Stream().cuda_stream)
+        hglib.hg_build_wedges(g, close_mode=2)
+        built = set(count.live)
+
+        def watch(live):
+            big.append(sum(1 for p, n in live.items() if p not in built and n > (4 << 20)))
+
+        count.on_change = watch
+        two = hglib.hg_count_patterns(g)
+        st = hglib.hg_close_stats_get(g)
+        count.on_change = None
+        hglib.hg_free(g)
+        assert not count.live
+    finally:
+        hglib.use_torch_allocator()
+    assert st["bucket_teams"][6] > 150   # both kinds were closed by the global-table teams
+    assert max(big) == 1, big
+    g = hglib.hg_load_csr(400, len(e_ptr) - 1, e_ptr, e_idx)
+    hglib.hg_build_wedges(g)
+    assert hglib.hg_count_patterns(g).tolist() == two.tolist()
+    hglib.hg_free(g)
