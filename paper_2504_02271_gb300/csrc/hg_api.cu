@@ -1100,14 +1100,33 @@ hg_status sample_impl(hg_graph* g, uint64_t seed, uint64_t first, uint64_t num, 
   return HG_OK;
 }
 
-// h_sel: NULL (every hyper-triangle), or one host byte per hyperedge: then only the
-// hyper-triangles owned by the hyperedges u with h_sel[u] != 0 (their teams alone run).
-hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nullptr) {
-  cudaStream_t s = g->stream;
-  release(g, g->count_blocks);
-  g->counted = g->have_cstats = false;
-  const int64_t ne = g->ne;
+// What a count decides before its teams start: the owners of every list, and the scratch.
+struct ClosePlan {
+  CloseLists cl;
+  TeamRule rule;
   Small h;
+  int32_t n[kLists];
+  int64_t slice_dmax = 0, slice = 0;   // the large bit-row teams' scratch: per block
+  int slice_blocks = 0;
+};
+
+// Scratch shape of global-table teams for out-degrees up to dmax and |e_u| up to smax.
+WideSpace wide_space(unsigned long long dmax, unsigned long long smax) {
+  WideSpace w;
+  w.dmax = std::max<int64_t>((int64_t)dmax, 1);
+  w.words = std::max<int64_t>(((int64_t)smax + 31) / 32, 1);
+  while (w.cap < 2 * w.dmax) w.cap *= 2;
+  return w;
+}
+
+size_t wide_bytes(const hg_graph* g, const WideSpace& w) {
+  return close_wide_scratch_bytes(w.cap, w.words, w.dmax, g->nsm);
+}
+
+// h_sel: see count_impl.
+hg_status plan_close(hg_graph* g, const uint8_t* h_sel, ClosePlan* p) {
+  cudaStream_t s = g->stream;
+  const int64_t ne = g->ne;
   // Arrays of |E| owners, two lists in each where no owner can be in both: bit-row classes from
   // both ends, a warp team's list and a block team's (bit-row teams append to these, but only
   // owners of their label), the two kinds of global-table teams, the handed-over owners.
@@ -1123,18 +1142,7 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
   HG_CUDA(cudaMemsetAsync(g->small->list_count, 0,
                           sizeof(g->small->list_count) + sizeof(g->small->label_count), s));
   HG_CUDA(cudaMemsetAsync(g->small->close_max, 0, sizeof(g->small->close_max), s));
-  HG_CUDA(cudaMemsetAsync(g->small->hist, 0, sizeof(g->small->hist), s));
-  HG_CUDA(cudaMemsetAsync(g->small->work, 0, sizeof(g->small->work), s));
-  HG_CUDA(cudaMemsetAsync(g->small->counters, 0, sizeof(int32_t) * 16, s));
-  // pattern bins: one set per member of a batch wave, else the handle's own
-  unsigned long long* hist = g->small->hist;
-  if (g->nm > 0) {
-    g->mhist = alloc_t<unsigned long long>(g, g->count_blocks, (int64_t)g->nm * 128);
-    if (!g->mhist) return HG_ERR_OOM;
-    HG_CUDA(cudaMemsetAsync(g->mhist, 0, sizeof(unsigned long long) * 128 * (size_t)g->nm, s));
-    hist = g->mhist;
-  }
-  CloseLists cl;
+  CloseLists& cl = p->cl;
   auto two_lists = [&](int array, int up, int down) {
     int32_t* base = lists + (int64_t)array * ne;
     cl.list[up] = OwnerList{base, 1, g->small->list_count + up};
@@ -1146,49 +1154,69 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
   for (int k = 0; k < kBitClasses; k += 2) two_lists(5 + k / 2, kListBits + k, kListBits + k + 1);
   cl.labels = g->small->label_count;
   cl.maxima = g->small->close_max;
-  DevGraph d = dev_graph(g);
-  TeamRule rule;
+  TeamRule& rule = p->rule;
   // the warp teams keep |e_x| in 16 bits: larger hyperedges send everything to the
   // global-table blocks
   rule.all_wide = g->close_mode == 1 || g->max_size >= 65536;
   rule.warp_max = g->warp_team_max;
   rule.block_max = g->packed ? kBlockMaxPacked : kBlockMaxUnpacked;
-  const int handover = g->close_mode == 2 ? 1 : 0;
   t_begin(g, "close_bucket");
-  launch_bucket_close(d, g->ori, cl, rule, sel, s);
+  launch_bucket_close(dev_graph(g), g->ori, cl, rule, sel, s);
   t_end(g);
-  HG_TRY(sync_small(g, &h));
-  int32_t n[kLists];
-  for (int k = 0; k < kLists; ++k) n[k] = h.list_count[k];
+  HG_TRY(sync_small(g, &p->h));
+  for (int k = 0; k < kLists; ++k) p->n[k] = p->h.list_count[k];
+  p->slice_dmax = ((int64_t)p->h.close_max[5] + 15) / 16 * 16;
+  p->slice = bits_slice_bytes(p->slice_dmax, (int64_t)p->h.close_max[4], g->nv);
+  p->slice_blocks = std::min(p->n[kListBits + kBitClasses - 1], g->nsm);
+  return HG_OK;
+}
+
+// h_sel: NULL (every hyper-triangle), or one host byte per hyperedge: then only the
+// hyper-triangles owned by the hyperedges u with h_sel[u] != 0 (their teams alone run).
+hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nullptr) {
+  cudaStream_t s = g->stream;
+  release(g, g->count_blocks);
+  g->counted = g->have_cstats = false;
+  const int64_t ne = g->ne;
+  HG_CUDA(cudaMemsetAsync(g->small->hist, 0, sizeof(g->small->hist), s));
+  HG_CUDA(cudaMemsetAsync(g->small->work, 0, sizeof(g->small->work), s));
+  HG_CUDA(cudaMemsetAsync(g->small->counters, 0, sizeof(int32_t) * 16, s));
+  // pattern bins: one set per member of a batch wave, else the handle's own
+  unsigned long long* hist = g->small->hist;
+  if (g->nm > 0) {
+    g->mhist = alloc_t<unsigned long long>(g, g->count_blocks, (int64_t)g->nm * 128);
+    if (!g->mhist) return HG_ERR_OOM;
+    HG_CUDA(cudaMemsetAsync(g->mhist, 0, sizeof(unsigned long long) * 128 * (size_t)g->nm, s));
+    hist = g->mhist;
+  }
+  ClosePlan plan;
+  HG_TRY(plan_close(g, h_sel, &plan));
+  const CloseLists& cl = plan.cl;
+  const int32_t* n = plan.n;
+  Small& h = plan.h;
   // scratch of the global-table teams: out-degrees and |e_u| up to the two maxima
-  auto wide_scratch = [&](unsigned long long dmax, unsigned long long smax, WideSpace* w) {
-    WideSpace need;
-    need.dmax = std::max<int64_t>((int64_t)dmax, 1);
-    need.words = std::max<int64_t>(((int64_t)smax + 31) / 32, 1);
-    while (need.cap < 2 * need.dmax) need.cap *= 2;
-    if (w->scratch) {   // of an earlier launch: kept when it is large enough
-      if (w->cap >= need.cap && w->words >= need.words && w->dmax >= need.dmax) return true;
-      release_one(g, g->count_blocks, w->scratch);
-    }
-    *w = need;
-    w->scratch = dev_alloc(g, g->count_blocks,
-                           close_wide_scratch_bytes(w->cap, w->words, w->dmax, g->nsm));
-    return w->scratch != nullptr;
-  };
   WideSpace wide;
-  const int64_t slice_dmax = ((int64_t)h.close_max[5] + 15) / 16 * 16;
-  const int64_t slice = bits_slice_bytes(slice_dmax, (int64_t)h.close_max[4], g->nv);
-  const int slice_blocks = std::min(n[kListBits + kBitClasses - 1], g->nsm);
+  auto wide_scratch = [&](unsigned long long dmax, unsigned long long smax) {
+    const WideSpace need = wide_space(dmax, smax);
+    if (wide.scratch) {   // of an earlier launch: kept when it is large enough
+      if (wide.cap >= need.cap && wide.words >= need.words && wide.dmax >= need.dmax) return true;
+      release_one(g, g->count_blocks, wide.scratch);
+    }
+    wide = need;
+    wide.scratch = dev_alloc(g, g->count_blocks, wide_bytes(g, wide));
+    return wide.scratch != nullptr;
+  };
   void* slices = nullptr;
-  if (slice_blocks > 0) {
-    slices = dev_alloc(g, g->count_blocks, (size_t)(slice * slice_blocks));
+  if (plan.slice_blocks > 0) {
+    slices = dev_alloc(g, g->count_blocks, (size_t)(plan.slice * plan.slice_blocks));
     if (!slices) return HG_ERR_OOM;
   }
   static const char* names[kLists] = {
       "close_warp256",  "close_warp512",   "close_warp1024",  "close_block2048", "close_block4096",
       "close_block8192", "close_wide",     "close_cluster",   "close_bits64",    "close_bits128",
       "close_bits256",  "close_bits512",   "close_bits1024",  "close_bits_large", "close_wide"};
-  const CloseRun run{d, g->ori, g->packed, hist, cl.list[kListOver], handover, s, g->nsm};
+  const int handover = g->close_mode == 2 ? 1 : 0;
+  const CloseRun run{dev_graph(g), g->ori, g->packed, hist, cl.list[kListOver], handover, s, g->nsm};
   ReturnLists ret;
   for (int k = 0; k < kCloseBuckets; ++k) ret.back[k] = cl.list[k];
   int64_t n_bits = 0;
@@ -1196,14 +1224,15 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
     if (n[k] <= 0) continue;
     n_bits += n[k];
     t_begin(g, names[k]);
-    HG_CUDA(launch_close_bits(k - kListBits, run, cl.list[k], n[k], ret, slices, slice, slice_dmax,
-                              slice_blocks, &g->small->work[0][0], rule, g->small->counters + k));
+    HG_CUDA(launch_close_bits(k - kListBits, run, cl.list[k], n[k], ret, slices, plan.slice,
+                              plan.slice_dmax, plan.slice_blocks, &g->small->work[0][0], plan.rule,
+                              g->small->counters + k));
     t_end(g);
   }
   // A walking team's list and what the bit-row teams gave back to it (`most`: an upper bound).
   auto walk = [&](int k, int64_t most) {
     if (k >= kListWide && k <= kListCluster &&
-        !wide_scratch(h.close_max[0], h.close_max[1], &wide))
+        !wide_scratch(h.close_max[0], h.close_max[1]))
       return HG_ERR_OOM;
     t_begin(g, names[k]);
     HG_CUDA(launch_close(k, run, cl.list[k], (int32_t)std::min<int64_t>(most, ne), wide,
@@ -1225,7 +1254,7 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
   if (n_over > 0) {
     // (the teams before are done: their scratch is reused or given back)
     if (slices) release_one(g, g->count_blocks, slices);
-    if (!wide_scratch(h.close_max[2], h.close_max[3], &wide)) return HG_ERR_OOM;
+    if (!wide_scratch(h.close_max[2], h.close_max[3])) return HG_ERR_OOM;
     HG_TRY(walk(kListOver, n_over));
     HG_TRY(sync_small(g, &h));
   }
@@ -2040,4 +2069,26 @@ hg_status hg_kernel_times(hg_graph* g, const char** names, float* ms, int32_t* l
 
 namespace hg {
 void alloc_bypass_hooks(bool on) { t_bypass_hooks = on; }
+
+hg_status handle_bytes(hg_graph* g, HandleBytes* out) {
+  *out = HandleBytes{};
+  if (!g->built) return HG_ERR_STATE;
+  for (const auto* owner : {&g->load_blocks, &g->build_blocks})
+    for (const Block& b : *owner) {
+      out->held += b.bytes;
+      if (g->packed && (b.p == g->cap_rows.packed || b.p == g->ori.packed)) out->packed_rows += b.bytes;
+    }
+  release(g, g->count_blocks);
+  g->counted = g->have_cstats = false;
+  ClosePlan plan;
+  const hg_status st = plan_close(g, nullptr, &plan);
+  if (st == HG_OK) {
+    for (const Block& b : g->count_blocks) out->count += b.bytes;
+    out->count += (size_t)(plan.slice * plan.slice_blocks);
+    if (plan.h.label_count[kWideBucket] + plan.h.label_count[kClusterBucket] > 0)
+      out->count += wide_bytes(g, wide_space(plan.h.close_max[0], plan.h.close_max[1]));
+  }
+  release(g, g->count_blocks);
+  return st;
+}
 }  // namespace hg

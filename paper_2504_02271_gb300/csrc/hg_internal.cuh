@@ -180,6 +180,13 @@ void launch_filter_rows(int keep, bool count_only, const int64_t* src_ptr, const
 
 // hg_api.cu: allocations of the calling thread skip the caller-installed hooks
 void alloc_bypass_hooks(bool on);
+// Device memory of a built handle: what it holds, how much of that is rows of packed entries
+// (twice as large unpacked), and what a count of it would take beside.  The last finds the
+// owners of every closure list on the device; a count made before is forgotten.
+struct HandleBytes {
+  size_t held = 0, packed_rows = 0, count = 0;
+};
+hg_status handle_bytes(hg_graph* g, HandleBytes* out);
 
 // k_batch.cu
 void launch_sub_base(int64_t* e_ptr, int32_t ne, int64_t base, cudaStream_t s);

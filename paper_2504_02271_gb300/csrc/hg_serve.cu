@@ -82,16 +82,14 @@ size_t bytes_of(const hg_server* S, const hg_query& q) {
   return is_exact(q) ? g.exact_bytes : g.sample_bytes;
 }
 
-// Device memory of one evaluation: inputs and transposes, step one (rows, degrees,
-// oriented entries over all 2W slots), step two (team lists, scratch), with slack.
-void size_graph(ServeGraph& g, int packed) {
-  const size_t ne = (size_t)g.ne, nv = (size_t)g.nv, nnz = (size_t)g.nnz, W = (size_t)g.W;
-  const size_t load = 16 * nnz + 40 * ne + 16 * nv;
-  const size_t build = 48 * ne + (packed ? 4 : 8) * 2 * W;
-  const size_t count = 32 * ne;
-  const size_t slack = size_t(64) << 20;
-  g.exact_bytes = load + build + count + slack;
-  g.sample_bytes = load + build + 8 * ne + (packed ? 4 : 8) * W + slack;
+// Device memory of one evaluation from what a handle of the hypergraph holds and would take:
+// rows of packed entries count twice (a batch with larger members is not packed), an estimate
+// adds the sorted rows (W entries, their offsets and index), and there is some slack.
+void size_graph(ServeGraph& g, const hg::HandleBytes& m) {
+  const size_t ne = (size_t)g.ne, W = (size_t)g.W;
+  const size_t built = m.held + m.packed_rows, slack = size_t(64) << 20;
+  g.exact_bytes = built + m.count + slack;
+  g.sample_bytes = built + 20 * ne + 8 * W + slack;
 }
 
 // Take the oldest query and what can join it (the caller holds the lock).
@@ -336,13 +334,18 @@ hg_status hg_server_add_graph(hg_server* S, int32_t num_vertices, int32_t num_ed
       (g.nnz > 0 && cudaMemcpy(g.d_idx, edge_vtx, sizeof(int32_t) * (size_t)g.nnz, kind) !=
                         cudaSuccess))
     st = HG_ERR_CUDA;
-  // validate and measure once: step one gives W for the memory estimates
+  // validate and measure once: a built handle gives W and the memory of an evaluation
+  hg::HandleBytes held;
   if (st == HG_OK) {
     hg::alloc_bypass_hooks(true);
     hg_graph* h = nullptr;
     hg_wedge_stats ws{};
     st = hg_load_csr(num_vertices, num_edges, g.d_ptr, g.d_idx, 1, nullptr, &h);
     if (st == HG_OK) st = hg_build_wedges(h, nullptr, &ws);
+    if (st == HG_OK) {
+      st = hg::handle_bytes(h, &held);
+      if (st == HG_ERR_OOM) st = HG_OK;   // no room for a count now: its lists are not measured
+    }
     if (h) hg_free(h);
     hg::alloc_bypass_hooks(false);
     g.W = ws.W;
@@ -352,7 +355,7 @@ hg_status hg_server_add_graph(hg_server* S, int32_t num_vertices, int32_t num_ed
     cudaFree(g.d_idx);
     return st;
   }
-  size_graph(g, 0);   // unpacked entries: an upper bound
+  size_graph(g, held);
   std::lock_guard<std::mutex> lk(S->mu);
   *graph_id = (int32_t)S->graphs.size();
   S->graphs.push_back(g);

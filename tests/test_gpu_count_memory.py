@@ -65,3 +65,43 @@ def test_one_scratch_of_the_global_table_teams_at_a_time(hglib):
     hglib.hg_build_wedges(g)
     assert hglib.hg_count_patterns(g).tolist() == two.tolist()
     hglib.hg_free(g)
+
+
+@pytest.mark.parametrize("shape", ["long", "coauthor", "tag"])
+def test_server_admits_by_what_an_evaluation_takes(hglib, shape):
+    # the bytes that the server books for a query against the peak of the same calls on a handle
+    # of the same hypergraph (the long shape has the 8-byte row layout)
+    from dataclasses import replace
+
+    import hgen
+    import torch
+
+    spec = {"long": replace(hgen.TAG_HEAVY, num_edges=12_000, num_vertices=20_000, size_p1=2.5,
+                            size_hi=600, degree_cap=100),
+            "coauthor": replace(hgen.COAUTHOR, num_edges=31_000, num_vertices=6_200),
+            "tag": replace(hgen.TAG_HEAVY, num_edges=5_000)}[shape]
+    e_ptr, e_idx = hgen.generate(spec)
+    nv, ne = spec.num_vertices, len(e_ptr) - 1
+    booked, peak = [], []
+    for kind in (hglib.HG_Q_COUNTS, hglib.HG_Q_ESTIMATE):
+        srv = hglib.Server(workers=1)
+        try:
+            gid = srv.add_graph(nv, e_ptr, e_idx)
+            assert srv.wait(srv.submit(kind, gid, seed=1, num_samples=1000))["status"] == 0
+            booked.append(srv.stats()["max_in_flight_bytes"])
+        finally:
+            srv.close()
+        count = Counting(hglib)
+        try:
+            g = hglib.hg_load_csr(nv, ne, e_ptr, e_idx, stream=torch.cuda.Stream().cuda_stream)
+            hglib.hg_build_wedges(g)
+            if kind == hglib.HG_Q_COUNTS:
+                hglib.hg_count_patterns(g)
+            else:
+                hglib.hg_sample_estimate(g, 1, 0, 1000)
+            hglib.hg_free(g)
+        finally:
+            hglib.use_torch_allocator()
+        peak.append(count.peak)
+    assert all(b >= p for b, p in zip(booked, peak)), (booked, peak)
+    assert booked[0] < 4 * peak[0] + (64 << 20)   # not so much that it admits nothing
