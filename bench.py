@@ -183,11 +183,8 @@ def source_sha(path):
         return hashlib.sha256(f.read()).hexdigest()[:16]
 
 
-def profiled_traffic(kernel, workload_name, units=None):
-    """DRAM bytes per launch from the committed ncu summary, if the kernel source is unchanged.
-
-    Entries captured on a smaller launch store bytes per unit (`dram_bytes_per_sample`);
-    they are scaled by the `units` of the measured launch."""
+def profiled(kernel, workload_name):
+    """The committed ncu summary of a kernel on a workload, if its source is unchanged."""
     path = os.path.join(ROOT, "profiles", "dram_traffic.json")
     try:
         with open(path) as f:
@@ -200,6 +197,17 @@ def profiled_traffic(kernel, workload_name, units=None):
     src = os.path.join(ROOT, "paper_2504_02271_gb300", "csrc", e["source"])
     if not os.path.exists(src) or source_sha(src) != e["source_sha"]:
         return None
+    return e
+
+
+def profiled_traffic(kernel, workload_name, units=None):
+    """DRAM bytes per launch from the committed ncu summary.
+
+    Entries captured on a smaller launch store bytes per unit (`dram_bytes_per_sample`);
+    they are scaled by the `units` of the measured launch."""
+    e = profiled(kernel, workload_name)
+    if e is None:
+        return None
     if "dram_bytes_per_sample" in e:
         return None if units is None else round(float(e["dram_bytes_per_sample"]) * units)
     return float(e["dram_bytes_per_launch"])
@@ -211,7 +219,7 @@ CLOSE_GROUPS = ("close_warp256", "close_warp512", "close_warp1024", "close_block
                 "close_block4096", "close_block8192", "close_bits64", "close_bits128",
                 "close_bits256", "close_bits512", "close_bits1024", "close_bits_large",
                 "close_wide", "close_cluster")
-ISSUE_LANE_OPS_PER_CYCLE_PER_SM = 4 * 32   # 4 schedulers, one 32-lane instruction per cycle
+ISSUE_SLOTS_PER_CYCLE_PER_SM = 4   # one warp instruction per scheduler and cycle
 
 
 def dram_rate(traffic, launch_ms, peak_gbs):
@@ -224,22 +232,60 @@ def dram_rate(traffic, launch_ms, peak_gbs):
                            " / live launch time"}
 
 
-def close_algorithmic(cs, T):
-    """Algorithmic work of the whole closure (all team shapes) in one pass.
+def list_walk_work(cs, T):
+    """What the list walk would do for the whole closure in one pass, whichever kernel closed
+    the hyperedges (bit rows answer the same probes without it).
 
     Per probe (an entry of out(v) looked up in u's table): 4 bytes read, 8 integer
     operations (decode 2, two hashes 2, two slot compares 4).  Per out-entry of u:
     20 bytes (entry, row start, out-degree, |e_x|) and 10 operations (table insert).
     Per E_y entry read for the vertex masks: 4 bytes and 8 operations.  Per
     hyper-triangle: 27 operations (index and mask loads 5, seven region tests 20,
-    histogram 2).  These are the list walk's operations; the bit-row teams answer the same
-    probes with fewer, so they are the yardstick there, not a count of what is executed.
-    """
+    histogram 2)."""
     probes, gathers, outs = cs["probes"], cs["gathers"], cs["out_entries"]
-    hits = T
-    nbytes = 4 * probes + 20 * outs + 4 * gathers
-    ops = 8 * probes + 10 * outs + 8 * gathers + 27 * hits
-    return nbytes, ops
+    return {"bytes": int(4 * probes + 20 * outs + 4 * gathers),
+            "ops": int(8 * probes + 10 * outs + 8 * gathers + 27 * T),
+            "note": "work of looking every entry of out(v) up, per step; the bit-row teams do not"
+                    " execute it"}
+
+
+def closure_roofline(kernel_ms, cs, T, clk, steps, workload_name):
+    """Issue and DRAM rates of the closure's kernels.
+
+    kernel_ms holds (summed ms, launches) over `steps` steps.  Executed instructions and DRAM
+    bytes per launch come from the committed captures of the kernels whose source is unchanged
+    (each launch of a workload does the same work); times are live.  Without a capture there is
+    no rate.  `covers` is the share of the closure's time that the captured kernels take."""
+    peak_hbm, peak_kind = measured_peaks()
+    groups = {n: v for n, v in kernel_ms.items() if n in CLOSE_GROUPS}
+    close_ms = sum(v[0] for v in groups.values()) / steps   # one step's closure
+    dom = max(groups, key=lambda n: groups[n][0])
+    sm_mhz = ((clk or {}).get("sm_mhz") or 2070.0)
+    peak = 152 * ISSUE_SLOTS_PER_CYCLE_PER_SM * sm_mhz * 1e6 / 1e12   # T warp instructions/s
+    ms = inst = dram = 0.0
+    for n, (total, launches) in groups.items():
+        e = profiled(n, workload_name)
+        if e is None or "inst_executed_per_launch" not in e:
+            continue
+        ms += total / steps
+        inst += float(e["inst_executed_per_launch"]) * launches / steps
+        dram += float(e["dram_bytes_per_launch"]) * launches / steps
+    rate = inst / (ms / 1000.0) / 1e12 if ms else None
+    hbm = dram_rate(dram, ms, peak_hbm)
+    return {"bound": "issue", "kernel": f"closure; {dom} is its largest kernel",
+            "achieved": None if rate is None else round(rate, 4), "peak": round(peak, 4),
+            "unit": "T warp instructions/s", "frac": None if rate is None else round(rate / peak, 4),
+            "peak_source": f"derived: 152 SMs x 4 issue slots/cycle x {sm_mhz:.0f} MHz (median SM"
+                           " clock under load)",
+            "source": "ncu smsp__inst_executed and dram__bytes of the committed captures / live"
+                      " time of the captured kernels",
+            "covers": round(ms / close_ms, 4) if close_ms else 0.0,
+            "closure_ms_per_step": round(close_ms, 4),
+            "launch_ms": round(groups[dom][0] / groups[dom][1], 4),
+            "traffic": round(dram) if hbm else None,
+            "hbm": {"achieved": hbm.get("dram_achieved"), "peak": peak_hbm, "unit": "GB/s",
+                    "frac": hbm.get("dram_frac"), "peak_source": peak_kind},
+            "list_walk": list_walk_work(cs, T)}
 
 
 # ------------------------------------------------------------------ multi-rank aggregation
@@ -402,27 +448,7 @@ def run_ours(args):
             dist.destroy_process_group()
         return
 
-    # roofline of the closure (its kernel with the largest share is named)
-    peak_hbm, peak_kind = measured_peaks()
-    groups = {n: v for n, v in kernel_ms.items() if n in CLOSE_GROUPS}
-    dom = max(groups, key=lambda n: groups[n][0])
-    dom_ms = groups[dom][0] / groups[dom][1]            # average launch duration
-    close_ms = sum(v[0] for v in groups.values()) / args.steps   # one step's closure
-    nbytes, ops = close_algorithmic(cs, int(counts[0]))
-    sm_mhz = ((clk or {}).get("sm_mhz") or 2070.0)
-    peak_ops = 152 * ISSUE_LANE_OPS_PER_CYCLE_PER_SM * sm_mhz * 1e6 / 1e12   # Tops/s
-    achieved_ops = ops / (close_ms / 1000.0) / 1e12
-    achieved_gbs = nbytes / (close_ms / 1000.0) / 1e9
-    traffic = profiled_traffic(dom, cfg["workload"])
-    roof = {"bound": "alu", "kernel": f"closure, all its kernels; {dom} is the largest",
-            "achieved": round(achieved_ops, 3), "peak": round(peak_ops, 2), "unit": "Tops/s",
-            "frac": round(achieved_ops / peak_ops, 4),
-            "peak_source": f"derived: 152 SMs x 128 lane-ops/cycle x {sm_mhz:.0f} MHz (median SM clock under load)",
-            "algorithmic_ops_per_step": int(ops), "algorithmic_bytes_per_step": int(nbytes),
-            "closure_ms_per_step": round(close_ms, 4), "launch_ms": round(dom_ms, 4), "traffic": traffic,
-            "hbm": {"achieved": round(achieved_gbs, 1), "peak": peak_hbm, "unit": "GB/s",
-                    "frac": round(achieved_gbs / peak_hbm, 4), "peak_source": peak_kind}}
-    roof["hbm"].update(dram_rate(traffic, dom_ms, peak_hbm))
+    roof = closure_roofline(kernel_ms, cs, int(counts[0]), clk, args.steps, cfg["workload"])
 
     dense = None
     if "dense_omega" in kernel_ms and st["dense_edges"]:
@@ -489,30 +515,6 @@ def run_ours(args):
 
 
 # ------------------------------------------------------------------ batches of hypergraphs
-
-def roofline_from_times(kernel_ms, cs, T, clk, steps):
-    """ALU roofline of the closure, all its kernels together (see close_algorithmic).
-
-    kernel_ms holds (summed ms, launches) over `steps` steps; cs and T are one step's work."""
-    peak_hbm, peak_kind = measured_peaks()
-    groups = {n: v for n, v in kernel_ms.items() if n in CLOSE_GROUPS}
-    dom = max(groups, key=lambda n: groups[n][0])
-    dom_ms = groups[dom][0] / groups[dom][1]            # average launch duration
-    close_ms = sum(v[0] for v in groups.values()) / steps   # one step's closure
-    nbytes, ops = close_algorithmic(cs, T)
-    sm_mhz = ((clk or {}).get("sm_mhz") or 2070.0)
-    peak_ops = 152 * ISSUE_LANE_OPS_PER_CYCLE_PER_SM * sm_mhz * 1e6 / 1e12
-    achieved_ops = ops / (close_ms / 1000.0) / 1e12
-    achieved_gbs = nbytes / (close_ms / 1000.0) / 1e9
-    return {"bound": "alu", "kernel": f"closure, all its kernels; {dom} is the largest",
-            "achieved": round(achieved_ops, 3), "peak": round(peak_ops, 2), "unit": "Tops/s",
-            "frac": round(achieved_ops / peak_ops, 4),
-            "peak_source": f"derived: 152 SMs x 128 lane-ops/cycle x {sm_mhz:.0f} MHz (median SM clock under load)",
-            "algorithmic_ops_per_step": int(ops), "algorithmic_bytes_per_step": int(nbytes),
-            "closure_ms_per_step": round(close_ms, 4), "launch_ms": round(dom_ms, 4), "traffic": None,
-            "hbm": {"achieved": round(achieved_gbs, 1), "peak": peak_hbm, "unit": "GB/s",
-                    "frac": round(achieved_gbs / peak_hbm, 4), "peak_source": peak_kind}}
-
 
 def run_batched(args):
     """4,096 independent hypergraphs (|E| log-uniform in [100, 200000], |V| = |E|/4,
@@ -657,7 +659,7 @@ def run_batched(args):
         e2e_ms.append(ms)
     e2e_value = T * len(e2e_ms) / (sum(e2e_ms) / 1000.0)
 
-    roof = roofline_from_times(kernel_ms, cs, T, clk, args.steps)
+    roof = closure_roofline(kernel_ms, cs, T, clk, args.steps, "batched")
     cpu = None
     if not args.skip_cpu_baseline:
         import oracle
