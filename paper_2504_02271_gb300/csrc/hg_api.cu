@@ -1206,11 +1206,13 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
     wide.scratch = dev_alloc(g, g->count_blocks, wide_bytes(g, wide));
     return wide.scratch != nullptr;
   };
+  // the large bit-row teams' scratch: on fewer blocks when there is no room for all
   void* slices = nullptr;
-  if (plan.slice_blocks > 0) {
-    slices = dev_alloc(g, g->count_blocks, (size_t)(plan.slice * plan.slice_blocks));
-    if (!slices) return HG_ERR_OOM;
-  }
+  int slice_blocks = plan.slice_blocks;
+  while (slice_blocks > 0 &&
+         !(slices = dev_alloc(g, g->count_blocks, (size_t)(plan.slice * slice_blocks))))
+    slice_blocks /= 2;
+  if (plan.slice_blocks > 0 && !slices) return HG_ERR_OOM;
   static const char* names[kLists] = {
       "close_warp256",  "close_warp512",   "close_warp1024",  "close_block2048", "close_block4096",
       "close_block8192", "close_wide",     "close_cluster",   "close_bits64",    "close_bits128",
@@ -1225,7 +1227,7 @@ hg_status count_impl(hg_graph* g, uint64_t counts[21], const uint8_t* h_sel = nu
     n_bits += n[k];
     t_begin(g, names[k]);
     HG_CUDA(launch_close_bits(k - kListBits, run, cl.list[k], n[k], ret, slices, plan.slice,
-                              plan.slice_dmax, plan.slice_blocks, &g->small->work[0][0], plan.rule,
+                              plan.slice_dmax, slice_blocks, &g->small->work[0][0], plan.rule,
                               g->small->counters + k));
     t_end(g);
   }

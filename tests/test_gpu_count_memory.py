@@ -15,8 +15,11 @@ class Counting:
 
         self.live, self.peak = {}, 0
         self.on_change = None
+        self.largest = None   # larger requests get no memory
 
         def alloc(nbytes, stream, _ctx):
+            if self.largest is not None and nbytes > self.largest:
+                return None
             p = torch.cuda.caching_allocator_alloc(int(nbytes), torch.cuda.current_device(),
                                                    int(stream or 0))
             self.live[p] = int(nbytes)
@@ -105,3 +108,24 @@ def test_server_admits_by_what_an_evaluation_takes(hglib, shape):
         peak.append(count.peak)
     assert all(b >= p for b, p in zip(booked, peak)), (booked, peak)
     assert booked[0] < 4 * peak[0] + (64 << 20)   # not so much that it admits nothing
+
+
+def test_bit_rows_on_fewer_blocks_when_memory_is_short(hglib):
+    # column lists of 130,000 entries per block: no room for a slice of scratch on every SM
+    import torch
+
+    edges = random_edges(3000, 1300, 90, 110, 9)
+    e_ptr, e_idx = csr_of(edges)
+    count = Counting(hglib)
+    try:
+        g = hglib.hg_load_csr(3000, len(e_ptr) - 1, e_ptr, e_idx,
+                              stream=torch.cuda.Stream().cuda_stream)
+        hglib.hg_build_wedges(g)
+        want = hglib.hg_count_patterns(g)
+        assert max(count.live.values()) > (12 << 20)   # a slice for each of up to 152 blocks
+        count.largest = 3 << 20
+        got = hglib.hg_count_patterns(g)
+        hglib.hg_free(g)
+    finally:
+        hglib.use_torch_allocator()
+    assert got.tolist() == want.tolist()
