@@ -18,15 +18,17 @@
 // set.  Classes without inclusion (9-20, nearly all) are counted by population counts of
 // 12 bit expressions; a pair with an inclusion is put in its labelled-mask bin by itself.
 //
-// Work per out-neighbour: its |e_v| vertices (one dictionary access each) and |e_v| words
-// per 32 out-neighbours, against one hash lookup and about 71 lane instructions per entry of
-// out(v) for the list walk that this replaces (95 entries of out(v) per out-neighbour on the
-// co-authorship workload, 1,350 on the tag-shaped prefix of 40,000 hyperedges).  The closure
-// there went from 8.0 to 6.0 ms and from 145 to 46 ms, on 2,000 uniform hyperedges over 1,000
-// vertices from 2.2 to 0.5 ms.  The small teams are bound by instruction issue and their
-// barriers (10,000-20,000 warp instructions a team), the large ones by the shared-memory
-// reads of the column words (half of their time) and by the vertices read from memory (a
-// third).
+// Work per out-neighbour v: its |e_v| vertices (one dictionary access each), and per 32
+// out-neighbours |e_u| words of e_u's columns and one word per shared vertex of e_v outside e_u,
+// against one hash lookup and about 71 lane instructions per entry of out(v) for the list walk
+// (95 entries of out(v) per out-neighbour on the co-authorship workload, 1,350 on the tag-shaped
+// prefix of 40,000 hyperedges).  The closure there went from 8.0 to 6.0 ms and from 145 to 46
+// ms, on 2,000 uniform hyperedges over 1,000 vertices from 2.2 to 0.5 ms.  Owners whose
+// neighbourhoods are sparse, or large hyperedges over few others, walk (list_of in
+// k_close.cu); an owner whose tables overflow goes back to the walking team of its shape.  The
+// small teams are bound by instruction issue and their barriers (10,000-20,000 warp
+// instructions a team), the large ones by the shared-memory reads of the column words (half of
+// their time) and by the vertices read from memory (a third).
 #include <type_traits>
 
 #include "hg_internal.cuh"

@@ -45,7 +45,7 @@ __device__ __forceinline__ void philox4x32_10(uint32_t c[4], uint32_t k0, uint32
 // memory (keys as stored in the packed layout, j << 32 | omega otherwise; padded to a power
 // of two).  A block per row spent its time in barriers and held 128 KB for about 40 entries:
 // an estimate on half of 150,000 co-authorship hyperedges, 1.33 ms of it this sort, went from
-// 3.50 to 2.41 ms.
+// 3.50 to 2.41 ms (2.2 with the longer rows dealt out as below).
 constexpr int kWarpSort = 512;
 
 template <bool PACKED>
@@ -212,7 +212,7 @@ __device__ int triple_common(const int32_t* a, int na, const int32_t* b, int nb,
 // queued, so that the loads of e_k run with every lane at work (a quarter of the candidates
 // of a co-authorship draw are hits), eight independent ones at a time.  On 500,000
 // co-authorship hyperedges 4 million draws went from 8.58 to 7.38 ms, 2 million of Algorithm 7
-// from 10.6 to 8.9; a listing over 50,000 hyperedges from 7.2 to 6.5.
+// from 10.6 to 8.8; a listing over 50,000 hyperedges from 7.2 to 6.5.
 
 constexpr int kCacheEntries = 384;   // searched rows up to this long go to shared memory
 constexpr int kCommonMax = 64;       // e_i cap e_j up to this large goes to shared memory

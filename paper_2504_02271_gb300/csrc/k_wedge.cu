@@ -82,13 +82,13 @@ __device__ __forceinline__ void ht_add(typename GatherSlot<PACKED>::T* T, int ca
   }
 }
 
-// Row i of a heavy hyperedge: its heavy neighbours come from the dense tiles, so the
-// gather skips them; light rows (and a graph without a dense path) gather everything.
-// heavy positions row i's tiles were multiplied for: its member's in a batch, else all
+// Heavy positions that row i's tiles were multiplied for: its member's in a batch, else all.
 __device__ __forceinline__ int2 heavy_range(const DevGraph& g, const DenseInfo& dn, int32_t i) {
   return dn.hrange ? dn.hrange[member_of(g, i)] : make_int2(0, dn.nh);
 }
 
+// Row i of a heavy hyperedge: its heavy neighbours come from the dense tiles, so the
+// gather skips them; light rows (and a graph without a dense path) gather everything.
 __device__ __forceinline__ bool gather_pair(const DenseInfo& dn, int32_t hi, int32_t j) {
   return hi < 0 || dn.heavy_idx[j] < 0;
 }
