@@ -88,3 +88,19 @@ def test_sparse_owners_with_long_neighbours_go_to_the_block_teams(hglib):
     check_against_oracle(hglib, 41_000, e_ptr, e_idx)
     _, kernels = closed_by(hglib, 41_000, e_ptr, e_idx)
     assert "close_block2048" in kernels
+
+
+@pytest.mark.parametrize("ne", [1201, 3001])
+def test_unpacked_block_teams(hglib, ne):
+    # the same star beside one hyperedge of 300 vertices that gives the two-array row layout:
+    # block teams of that layout up to out-degree 4,096
+    first, nv = 300_000, 40_000
+    e_ptr, e_idx = star(nv, ne, 24, ne, first)
+    e_ptr = np.concatenate([e_ptr, [e_ptr[-1] + 300]]).astype(np.int64)
+    e_idx = np.concatenate([e_idx, np.arange(300, dtype=np.int32)])
+    counts, st = gpu_count(hglib, first + nv, e_ptr, e_idx)
+    wide, ws = gpu_count(hglib, first + nv, e_ptr, e_idx, close_mode=1)
+    assert int(counts[0]) == ne * (ne - 1) * (ne - 2) // 6
+    assert counts.tolist() == wide.tolist() and st["masks"] == ws["masks"]
+    _, kernels = closed_by(hglib, first + nv, e_ptr, e_idx)
+    assert ("close_block8192" if ne > 2048 else "close_block2048") in kernels
